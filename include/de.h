@@ -184,7 +184,12 @@ int de_step(de_ctx *ctx);
  * with its own stream are captured once per distinct count into a CUDA graph
  * (on the first run of that count, or by de_prepare_run) and replayed; a
  * setter that changes the launch (kernel, launch shape, pipeline, base rule,
- * wait limit) drops the cached graphs. */
+ * wait limit) drops the cached graphs. Populations that the GPU's shared
+ * memory holds advance many generations per launch, with the results of
+ * de_step bit for bit; the first such run takes two more population buffers
+ * from the allocator (without them, and on a capturing stream, every
+ * generation is a launch). The waits between rows in that launch give up
+ * after 1 s (DE_ETIMEOUT). */
 int de_run(de_ctx *ctx, int32_t generations);
 
 /* Capture and instantiate the graph that de_run(ctx, generations) replays,

@@ -395,17 +395,69 @@ int de_step(de_ctx* c) {
   return rc;
 }
 
+// Whether runs of this context go through the resident kernel: rows of the
+// row-per-CTA kernel chosen automatically, a base rule that needs nothing from
+// the previous generation's close, and a population that the chip holds. The
+// first such run takes the kernel's buffers; if that fails, runs launch each
+// generation.
+static bool resident_ready(de_ctx* c, ResidentShape* shape) {
+  if (c->batch || c->rotated || c->use_pipe || c->use_stream || c->kernel_req != 0) return false;
+  if (c->p.base == kBaseBest) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+  const bool ok = prepare_resident(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR, c->sm_count,
+                                   c->smem_optin, shape);
+  cudaGetLastError();
+  if (!ok) return false;
+  if (c->res_state) return true;
+  ResState* rs = (ResState*)ctx_alloc(c, sizeof(ResState));
+  uint32_t* words = (uint32_t*)ctx_alloc(c, (size_t)c->N * kResWordStride * sizeof(uint32_t));
+  float* pop2 = (float*)ctx_alloc(c, 2 * (size_t)c->N * (size_t)c->pitch * sizeof(float));
+  // row words and counters start at tag 0, the first launch at tag 8: no word
+  // is taken for one of its generations before its owner has written it
+  ResState s0;
+  std::memset(&s0, 0, sizeof(s0));
+  s0.epoch = 8u;
+  s0.hist = ~0ULL;
+  if (rs && words && pop2 && cudaMemcpyAsync(rs, &s0, sizeof(s0), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
+      cudaMemsetAsync(words, 0, (size_t)c->N * kResWordStride * sizeof(uint32_t), c->stream) == cudaSuccess) {
+    c->res_state = rs;
+    c->res_words = words;
+    c->res_pop2 = pop2;
+    return true;
+  }
+  cudaGetLastError();
+  for (void* q : {(void*)rs, (void*)words, (void*)pop2})
+    if (q) ctx_free(c, q);
+  return false;
+}
+
 // The cached graph of `generations` generations, captured and instantiated on
 // first use. Capture records launches without running them, so the context's
 // device state is unchanged; nullptr on a CUDA error.
 static cudaGraphExec_t run_graph(de_ctx* c, int32_t generations) {
   auto it = c->graphs.find(generations);
   if (it != c->graphs.end()) return it->second;
+  ResidentShape shape;
+  const bool resident = resident_ready(c, &shape);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return nullptr;
   cudaError_t le = cudaSuccess;
-  for (int32_t k = 0; k < generations && le == cudaSuccess; ++k) le = launch_generation(c, c->p);
+  if (resident) {
+    ResidentParams rp{};
+    rp.g = c->p;
+    rp.rs = c->res_state;
+    rp.words = c->res_words;
+    rp.pop2 = c->res_pop2;
+    rp.row_threads = c->block;
+    for (int32_t left = generations; left > 0 && le == cudaSuccess; left -= rp.gens) {
+      rp.gens = std::min(left, kResMaxGens);
+      le = launch_resident(c->xo, c->obj, c->vidx, shape, rp, c->stream);
+    }
+  } else {
+    for (int32_t k = 0; k < generations && le == cudaSuccess; ++k) le = launch_generation(c, c->p);
+  }
   e = cudaStreamEndCapture(c->stream, &graph);
   if (le != cudaSuccess || e != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);

@@ -43,6 +43,49 @@ cudaError_t prepare_gen_pipe(int xo, int obj, size_t smem);
 cudaError_t launch_gen_pipe(int xo, int obj, const PipeParams& pp, int grid, int block, size_t smem,
                             cudaStream_t s);
 
+// Resident generation kernel (gen_resident.cuh): many generations of a
+// population held on the chip in one cooperative launch.
+constexpr int kResWarps = 16, kResHelpers = 2, kResThreads = 32 * (kResWarps + kResHelpers);   // rows' warps, helper warps
+constexpr int kResWordStride = 32;   // a row word has a 128-byte line of its own
+// A launch makes at most this many generations, which bounds its time.
+constexpr int kResMaxGens = 4096;
+struct ResState {
+  unsigned epoch;              // row tag that the next launch starts at (tags do not repeat between launches)
+  unsigned pad_;
+  unsigned long long hist;     // (orderable best value of the run << 32) | first generation that reached it
+  unsigned pad2_[28];
+  unsigned ctr[8];             // CTAs that finished generation k, k mod 8, on a line of their own; zero between launches
+  unsigned pad3_[24];
+};
+struct ResidentParams {
+  GenParams g;
+  ResState* rs;
+  uint32_t* words;             // N row words, kResWordStride apart
+  float* pop2;                 // third and fourth buffer, N x pitch each
+  int gens;                    // generations of this launch
+  int rpc;                     // rows per CTA
+  int row_threads;             // threads per row in gen_kernel's order
+  int groups, xo;              // rows a CTA processes at a time; crossover
+};
+struct ResidentShape {
+  int grid, block, rpc, groups;
+  bool seg;                    // the kernel for segments
+  size_t smem;
+};
+// The launch shape for rows of block x kVecChoices[vidx] slots, and the
+// kernel's attributes set for it; false if the population does
+// not fit or a launch per generation is the faster.
+bool prepare_resident(int xo, int obj, int vidx, int block, int N, int D4, double CR, int sm_count, int smem_optin,
+                      ResidentShape* out);
+cudaError_t launch_resident(int xo, int obj, int vidx, const ResidentShape& sh, ResidentParams rp, cudaStream_t s);
+// seg: the kernel that computes what a segment changed, else whole rows
+const void* resident_entry_sphere(bool seg, int vidx);
+const void* resident_entry_rastrigin(bool seg, int vidx);
+const void* resident_entry_ackley(bool seg, int vidx);
+const void* resident_entry_rosenbrock(bool seg, int vidx);
+const void* resident_entry_griewank(bool seg, int vidx);
+const void* resident_entry_elliptic(bool seg, int vidx);
+
 // Batched instances (batch_kernel.cu): one descriptor per instance and a
 // tile list; a tile is 256 / group rows of one instance.
 struct alignas(16) BatchInst {  // copied into shared memory 16 bytes at a time
