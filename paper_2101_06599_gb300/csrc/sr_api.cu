@@ -117,6 +117,7 @@ int sr_setup(de_ctx* c, const de_objparams* prm) {
   c->rotated = true;
   sp.obj = c->obj;
   sp.prec = (prm->prec == DE_PREC_BF16) ? 2 : (prm->prec == DE_PREC_FP16 ? 3 : 0);
+  sp.sm_count = c->sm_count;
   sp.a_scale = 1.0f;
   sp.z_scale = 1.0f;
   sp.nct2 = (D + kSrTile - 1) / kSrTile;

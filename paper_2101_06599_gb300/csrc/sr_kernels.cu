@@ -231,114 +231,173 @@ __device__ __forceinline__ void sr_tile_reduce(const SrParams& sp, const float z
   }
 }
 
-// All rows (modes 0 and 1): 128 x 128 output tile, 256 threads, 8 rows x
-// (2 x 4) columns per thread (columns tx*4.. and 64 + tx*4.. so that each
-// 64-column half keeps the lane layout above), K in steps of 16 through a
-// double-buffered shared-memory stage with the next step prefetched into
-// registers. VEC: D % 4 == 0, 16-byte loads of x, o and R.
-constexpr int kGbM = 128, kGbN = 128, kGbK = 16, kGbLd = kGbM + 4;
+// All rows (modes 0 and 1): tiles of 8 RT rows x 64 columns, 128 threads, RT
+// rows x 4 columns per thread (thread tx of 16 has the columns 4 tx .. 4 tx + 3,
+// the lane layout above), K in steps of 16. x and R^T arrive two steps ahead
+// by cp.async (read one step ahead through registers, the loads were the first
+// stall); a step before its use each thread turns the x it copied itself into
+// a = fl(x - o), K-major.
+//
+// Bound by the FP32 pipe (2 N D^2 flop; 128 FMA per SM and clock, busy 67 % of
+// the time here, 50 % before) and, next, by shared-memory loads. The products
+// are fma.rn.f32x2 on pairs of rows: the same pipe rate in half the issue slots,
+// so that the shared loads and the operand copies issue beside them; each half is
+// its element's own fmaf chain over j ascending. N = 4096, D = 1024, a generation:
+// 271 us with 128 x 128 tiles of scalar FMAs (256 tiles: two on some SMs, one on
+// the others), 189 us with 592 tiles of 112 x 64, four on almost every SM.
+constexpr int kGbN = 64, kGbK = 16, kGbThreads = 128, kGbLdB = kGbN + 4;
 
-template <bool VEC>
-__global__ void __launch_bounds__(256, 2) sr_gemm_fp32_kernel(const __grid_constant__ SrParams sp, int mode) {
+__device__ __forceinline__ void ffma2(unsigned long long& c, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+  return v;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+
+// VEC: D % 4 == 0, 16-byte copies of x, o and R^T; else single elements.
+template <int RT, bool VEC>
+__global__ void __launch_bounds__(kGbThreads, 4) sr_gemm_fp32_kernel(const __grid_constant__ SrParams sp, int mode) {
   griddep_wait();                                  // the previous kernel of the generation is done
   griddep_launch_dependents();
+  static_assert(RT % 2 == 0 && RT >= 4 && RT <= 16, "pairs of rows");
+  constexpr int M = 8 * RT, LdA = M + 4, P = RT / 2, kQuads = RT / 4;
+  constexpr int kLoads = (M * 4 + kGbThreads - 1) / kGbThreads;   // four-element pieces of a step's rows per thread
   const GenParams& p = sp.g;
-  __shared__ __align__(16) float As[2][kGbK][kGbLd];
-  __shared__ __align__(16) float Bs[2][kGbK][kGbLd];
-  __shared__ const float* rowp[kGbM];
+  __shared__ __align__(16) float As[2][kGbK][LdA];
+  __shared__ __align__(16) float Bs[3][kGbK][kGbLdB];
+  __shared__ __align__(16) float4 Xs[2][kLoads][kGbThreads];
+  __shared__ __align__(16) float Os[4][kGbK];
+  __shared__ const float* rowp[M];
 
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int n0 = blockIdx.x * kGbN, r0 = blockIdx.y * kGbM;
+  const int n0 = blockIdx.x * kGbN, r0 = blockIdx.y * M;
   const long long gen = p.st->gen;
   const uint8_t* slot_in = p.slots + (size_t)(gen & 1) * p.N;
-  if (t < kGbM) rowp[t] = (r0 + t < p.N) ? sr_row_ptr(sp, mode, r0 + t, slot_in) : nullptr;
+  for (int m = t; m < M; m += kGbThreads) rowp[m] = (r0 + m < p.N) ? sr_row_ptr(sp, mode, r0 + m, slot_in) : nullptr;
   __syncthreads();
 
-  // loader: row / column lm of the tile, 8 consecutive k from lk
-  const int lm = t & (kGbM - 1), lk = (t >> 7) * 8;
-  const float* xa = rowp[lm];
-  const float* rb = (n0 + lm < p.D) ? sp.rot + (size_t)(n0 + lm) * p.D : nullptr;
-  float va[8], vb[8];
-  auto load = [&](int k0) {
-    const int j0 = k0 + lk;
-    if constexpr (VEC) {
+  // step k0 to stage `at` of x (two) and `bt` of R^T (three); past D: zeros.
+  // Four lanes copy a row's 16 elements, four each
+  const int ak = 4 * (t & 3);                      // this thread's elements of every row
+  auto issue = [&](int k0, int at, int bt) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int j = j0 + 4 * h;
-        float4 x4 = make_float4(0.f, 0.f, 0.f, 0.f), r4 = x4;
-        if (j < p.D) {
-          const float4 o4 = *reinterpret_cast<const float4*>(sp.shift + j);
-          if (xa) {
-            x4 = *reinterpret_cast<const float4*>(xa + j);
-            x4 = make_float4(__fsub_rn(x4.x, o4.x), __fsub_rn(x4.y, o4.y), __fsub_rn(x4.z, o4.z), __fsub_rn(x4.w, o4.w));
-          }
-          if (rb) r4 = *reinterpret_cast<const float4*>(rb + j);
+    for (int u = 0; u < kLoads; ++u) {
+      const int m = (t + kGbThreads * u) >> 2, j = k0 + ak;
+      const float* xa = m < M ? rowp[m] : nullptr;
+      const uint32_t dst = sr_smem_u32(&Xs[at][u][t]);
+      if constexpr (VEC) {
+        const bool in = xa && j < p.D;
+        cp_async16(dst, in ? xa + j : sp.shift, in ? 16u : 0u);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const bool in = xa && j + e < p.D;
+          cp_async4(dst + 4 * e, in ? xa + j + e : sp.shift, in ? 4u : 0u);
         }
-        va[4 * h + 0] = x4.x; va[4 * h + 1] = x4.y; va[4 * h + 2] = x4.z; va[4 * h + 3] = x4.w;
-        vb[4 * h + 0] = r4.x; vb[4 * h + 1] = r4.y; vb[4 * h + 2] = r4.z; vb[4 * h + 3] = r4.w;
-      }
-    } else {
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int j = j0 + u;
-        va[u] = (xa && j < p.D) ? __fsub_rn(xa[j], sp.shift[j]) : 0.0f;
-        vb[u] = (rb && j < p.D) ? rb[j] : 0.0f;
       }
     }
-  };
-  auto store = [&](int buf) {
+    constexpr int kW = VEC ? 4 : 1;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      As[buf][lk + u][lm] = va[u];
-      Bs[buf][lk + u][lm] = vb[u];
+    for (int u = 0; u < kGbK * kGbN / kW / kGbThreads; ++u) {
+      const int c = t + kGbThreads * u, k = c / (kGbN / kW), n = (c % (kGbN / kW)) * kW;
+      const bool in = k0 + k < p.D && n0 + n < p.D;
+      const float* src = in ? sp.rot_t + (size_t)(k0 + k) * p.D + n0 + n : sp.rot_t;
+      if constexpr (VEC) cp_async16(sr_smem_u32(&Bs[bt][k][n]), src, in ? 16u : 0u);
+      else cp_async4(sr_smem_u32(&Bs[bt][k][n]), src, in ? 4u : 0u);
+    }
+  };
+  // o of a step, three steps ahead: other threads read it, so it takes a barrier
+  // after it has landed
+  auto issue_o = [&](int step) {
+    if (t < kGbK) {
+      const bool in = step * kGbK + t < p.D;
+      cp_async4(sr_smem_u32(&Os[step & 3][t]), in ? sp.shift + step * kGbK + t : sp.shift, in ? 4u : 0u);
+    }
+  };
+  auto form_a = [&](int step, int at, int buf) {   // x and o are zero past D, and so is a
+    const float4 o = *reinterpret_cast<const float4*>(&Os[step & 3][ak]);
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int m = (t + kGbThreads * u) >> 2;
+      if (m >= M) continue;
+      const float4 x = Xs[at][u][t];
+      As[buf][ak + 0][m] = __fsub_rn(x.x, o.x);
+      As[buf][ak + 1][m] = __fsub_rn(x.y, o.y);
+      As[buf][ak + 2][m] = __fsub_rn(x.z, o.z);
+      As[buf][ak + 3][m] = __fsub_rn(x.w, o.w);
     }
   };
 
-  float acc[8][8];
+  // rows of thread ty: 32 i + 4 ty .. + 3 for i < RT / 4, then (RT = 4 i + 2)
+  // 32 i + 2 ty, + 1; acc holds them in pairs
+  unsigned long long acc[P][4];
 #pragma unroll
-  for (int a = 0; a < 8; ++a)
+  for (int a = 0; a < P; ++a)
 #pragma unroll
-    for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0ULL;
 
-  load(0);
-  store(0);
+  issue(0, 0, 0);
+  issue_o(0);
+  issue_o(1);
+  cp_async_commit();
+  if (kGbK < p.D) issue(kGbK, 1, 1);
+  issue_o(2);
+  cp_async_commit();
+  cp_async_wait<1>();
   __syncthreads();
-  int buf = 0;
-  for (int k0 = 0; k0 < p.D; k0 += kGbK) {
-    const bool more = k0 + kGbK < p.D;
-    if (more) load(k0 + kGbK);
+  form_a(0, 0, 0);
+  __syncthreads();
+  const int steps = (p.D + kGbK - 1) / kGbK;
+  int bt = 0;                                      // stage of R^T of this step
+  for (int step = 0; step < steps; ++step) {
+    const int buf = step & 1, bt2 = bt == 0 ? 2 : bt - 1;
+    if (step + 2 < steps) issue((step + 2) * kGbK, buf, bt2);   // both stages were read before the last barrier
+    issue_o(step + 3);
+    cp_async_commit();
 #pragma unroll
     for (int kk = 0; kk < kGbK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 8]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 8 + 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][64 + tx * 4]);
-      const float ar[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float br[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      unsigned long long a[P];
 #pragma unroll
-      for (int a = 0; a < 8; ++a)
+      for (int i = 0; i < kQuads; ++i) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&As[buf][kk][32 * i + 4 * ty]);
+        a[2 * i] = v.x;
+        a[2 * i + 1] = v.y;
+      }
+      if constexpr (RT % 4 == 2) a[P - 1] = *reinterpret_cast<const unsigned long long*>(&As[buf][kk][32 * kQuads + 2 * ty]);
+      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[bt][kk][4 * tx]);
+      const unsigned long long b[4] = {pack2(b4.x, b4.x), pack2(b4.y, b4.y), pack2(b4.z, b4.z), pack2(b4.w, b4.w)};
 #pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(ar[a], br[b], acc[a][b]);
+      for (int i = 0; i < P; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ffma2(acc[i][c], a[i], b[c]);
     }
-    if (more) store(buf ^ 1);
+    cp_async_wait<1>();                            // step + 1 has landed
+    if (step + 1 < steps) form_a(step + 1, buf ^ 1, buf ^ 1);
     __syncthreads();
-    buf ^= 1;
+    bt = bt == 2 ? 0 : bt + 1;
   }
+  cp_async_wait<0>();
 
-  float* pg = sp.part_g;
-  float* pw = sp.part_w;
 #pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const int e = r0 + ty * 8 + a;
+  for (int i = 0; i < P; ++i) {
+    const int m = (RT % 4 == 2 && i == P - 1) ? 32 * kQuads + 2 * ty : 32 * (i >> 1) + 4 * ty + 2 * (i & 1);
+    const float2 z0 = unpack2(acc[i][0]), z1 = unpack2(acc[i][1]), z2 = unpack2(acc[i][2]), z3 = unpack2(acc[i][3]);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const float z[4] = {acc[a][4 * h], acc[a][4 * h + 1], acc[a][4 * h + 2], acc[a][4 * h + 3]};
-      const int c0 = n0 + 64 * h;
+      const float z[4] = {h ? z0.y : z0.x, h ? z1.y : z1.x, h ? z2.y : z2.x, h ? z3.y : z3.x};
+      const int e = r0 + m + h;
       float sg, sw;
-      sr_tile_reduce(sp, z, c0 + tx * 4, sg, sw);
-      if (tx == 0 && e < p.N && c0 < p.D) {
-        pg[(size_t)e * sp.nct2 + (c0 >> 6)] = sg;
-        pw[(size_t)e * sp.nct2 + (c0 >> 6)] = sw;
+      sr_tile_reduce(sp, z, n0 + 4 * tx, sg, sw);
+      if (tx == 0 && e < p.N) {
+        sp.part_g[(size_t)e * sp.nct2 + blockIdx.x] = sg;
+        sp.part_w[(size_t)e * sp.nct2 + blockIdx.x] = sw;
       }
     }
   }
@@ -704,6 +763,16 @@ cudaError_t launch_sr_trial(int xo, int /*vidx*/, const SrParams& sp, int /*bloc
   return launch_pdl(sr_trial_kernel<kNec>, dim3(grid), dim3(kTrialWarps * 32), 0, s, sp);
 }
 
+template <int RT>
+static cudaError_t launch_gemm_rows(dim3 grid, bool vec, const SrParams& sp, int mode, cudaStream_t s) {
+  // Not with programmatic dependent launch: CTAs that start while the trial
+  // kernel still fills the SMs are placed where room is left, several to an SM
+  // and none on others, and stay there (N = 1000, D = 1024: 65 us alone, 130 us so).
+  if (vec) sr_gemm_fp32_kernel<RT, true><<<grid, kGbThreads, 0, s>>>(sp, mode);
+  else sr_gemm_fp32_kernel<RT, false><<<grid, kGbThreads, 0, s>>>(sp, mode);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_sr_gemm_fp32(const SrParams& sp, int mode, int max_rows, cudaStream_t s) {
   const unsigned gx = (unsigned)((sp.g.D + kGbN - 1) / kGbN);
   if (mode == 2) {                                // split-operand paths: D % 256 == 0
@@ -712,9 +781,31 @@ cudaError_t launch_sr_gemm_fp32(const SrParams& sp, int mode, int max_rows, cuda
     const int grid = std::max(1, std::min(sp.list_ctas, (items + kLsGroups - 1) / kLsGroups));
     return launch_pdl(sr_gemm_fp32_list_kernel, dim3((unsigned)grid), dim3(kLsThreads), kLsSmem, s, sp);
   }
-  const dim3 grid(gx, (unsigned)((max_rows + kGbM - 1) / kGbM));
-  if (sp.g.D % 4 == 0) return launch_pdl(sr_gemm_fp32_kernel<true>, grid, dim3(256), 0, s, sp, mode);
-  return launch_pdl(sr_gemm_fp32_kernel<false>, grid, dim3(256), 0, s, sp, mode);
+  // Rows per tile (8 RT): every SM works through ceil(tiles / SMs) of them, each
+  // taking about RT + 1.5 (the loads and copies of a step do not shrink with RT).
+  // us per generation by RT = 16, 14, 12, 8, 4: N = 4096, D = 1024 204, 190, 194,
+  // 191, 248; N = 1000, D = 512 47, 44, 38, 31, 31; N = 16384, D = 1024 657, 687,
+  // 646, 687, 921; N = 700, D = 300 34, 32, 28, 24, 20.
+  const int sms = sp.sm_count > 0 ? sp.sm_count : 1;
+  int best = 16;
+  double cost = 1e30;
+  for (int rt : {16, 14, 12, 8, 4}) {
+    const long long tiles = (long long)gx * ((max_rows + 8 * rt - 1) / (8 * rt));
+    const double c = (double)((tiles + sms - 1) / sms) * (rt + 1.5);
+    if (c < cost) {
+      cost = c;
+      best = rt;
+    }
+  }
+  const dim3 grid(gx, (unsigned)((max_rows + 8 * best - 1) / (8 * best)));
+  const bool vec = sp.g.D % 4 == 0;
+  switch (best) {
+    case 16: return launch_gemm_rows<16>(grid, vec, sp, mode, s);
+    case 14: return launch_gemm_rows<14>(grid, vec, sp, mode, s);
+    case 12: return launch_gemm_rows<12>(grid, vec, sp, mode, s);
+    case 8: return launch_gemm_rows<8>(grid, vec, sp, mode, s);
+    default: return launch_gemm_rows<4>(grid, vec, sp, mode, s);
+  }
 }
 
 cudaError_t launch_sr_select(const SrParams& sp, const SrBound& b, cudaStream_t s) {
