@@ -468,16 +468,16 @@ int de_get_pipeline(de_ctx *ctx, int32_t *consumer_threads, int32_t *stages, int
  *
  * One DE/rand/1/NEC generation on caller-owned device buffers; the call
  * allocates nothing (no cudaMalloc/cudaFree, no allocating library routine).
- * Its scratch (generation state, slot bytes, NEC thresholds; 256 + 2*65536 +
- * 4*32768 bytes) is a fixed array compiled into the library, held by every GPU
- * that loads the library until the process exits.
+ * Its scratch (the NEC thresholds, 4*32768 bytes) is a fixed array compiled
+ * into the library, held by every GPU that loads the library until the process
+ * exits.
  *   pop_in, pop_out: device, N rows of `pitch` floats (pitch >= D, a multiple
  *     of 4; both bases 16-byte aligned; distinct buffers); pop_in is read only.
  *   fit_in, fit_out: device, N floats (distinct buffers).
  *   Row i of pop_out / fit_out receives the trial and its FP32 fitness if the
  *   trial is strictly better than fit_in[i], else a copy of the parent row and
  *   fit_in[i]. Draws come from Philox with (seed, generation), as de_step's at
- *   that generation. For D < 2048 the call runs the kernel de_step runs, so
+ *   that generation. For D < 2048 the call sums as the kernel de_step runs, so
  *   pop_out and fit_out are bit-identical to what de_step computes from the
  *   same population; for D >= 2048 de_step's pipelined kernel sums the FP32
  *   fitness in another order, so fitness values may differ in the last bits
@@ -487,14 +487,12 @@ int de_get_pipeline(de_ctx *ctx, int32_t *consumer_threads, int32_t *stages, int
  * Limits: 4 <= N <= 65536, 1 <= D <= 32768; larger sizes return DE_EINVAL.
  * Work is queued on `cuda_stream`. The first call on a device looks up the
  * scratch array's device address (cudaGetSymbolAddress) with that device
- * current; make that first call before any stream capture. Every call reuses
- * the same scratch and clears what must start at zero. The NEC thresholds are
+ * current; make that first call before any stream capture. The NEC thresholds are
  * rebuilt only when (Cr, D) differ from the previous call's on the device:
  * a chain of up to D - 1 dependent FP64 products, shorter the smaller Cr is
  * (measured on GB300: about 1.5 ms at D = 32768 with Cr = 0.9999, 0.03 ms
  * at Cr = 0.9), which only that call pays; a call with the thresholds kept
- * costs 0.03-0.05 ms at these sizes. Calls
- * that overlap on the GPU (different streams or host threads) race on the
+ * is one kernel. Calls that overlap on the GPU (different streams or host threads) race on the
  * scratch and must be serialised by the caller. */
 int de_nec_step_noalloc(const float *pop_in, const float *fit_in, float *pop_out, float *fit_out,
                         int32_t N, int32_t D, int32_t pitch, float F, double CR, de_objective obj,
