@@ -244,10 +244,11 @@ def time_batched(DE, torch, steps, warmup, seed, peak, n_inst=None, kernels="tun
     return {"workload": "batched_512_instances" if len(specs) == 512 else "batched_first_%d_instances" % len(specs),
             "instances": len(specs), "ind_dims_per_step": units,
             "value": units * steps / (ms / 1e3), "unit": UNIT, "ms_per_gen": ms / steps,
-            "hbm_gbs": gbs, "frac": gbs / peak,
-            # every instance on the staged, or every one on the streaming kernel: one
-            # cooperative launch per generation
-            "launches_per_step": 1 if kinds in (["staged"], ["streaming"]) else 2 + len(kinds),
+            # a run keeps the rows' partial sums and touches only what the segments change, one
+            # launch per generation: the share that reading every row once would need
+            # at the copy rate, over 1 when a generation is faster than that
+            "full_rows_share": gbs / peak,
+            "launches_per_step": 1,
             "row_kernels": {kd: sum(1 for g in groups if kind(g) == kd) for kd in kinds},
             "autotune_s": round(t_tune, 3),
             "a_acceptance": d_acc / (rows * steps), "m_masked_fraction": d_msk / (units * steps)}

@@ -320,7 +320,12 @@ typedef struct {
  * de_step / de_run step advances every instance by one generation: one
  * cooperative kernel launch (draws, rows, close) when every instance is on
  * the staged kernel (the default for exp / NEC rows of D <= 2048), else a
- * few launches over all instances (draws, row kernels, close). The rows of
+ * few launches over all instances (draws, row kernels, close). A de_run of
+ * two or more generations on exp / NEC rows of D <= 2048 (1 / (1 - Cr) <= 60,
+ * no wait limit set) keeps the rows' partial sums for the run and touches only
+ * what the segments change, with the same results bit for bit; the first such
+ * run takes 128 to 384 bytes per row from the allocator (without them the run
+ * reads every row). The rows of
  * each instance are cut into spans of up to 32 rows (taken by warps from a
  * queue) or, for D > 2048, into tiles of 256 / G rows; the row kernel of
  * each instance is set by de_batch_set_groups or de_batch_autotune. A device

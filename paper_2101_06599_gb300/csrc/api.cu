@@ -439,7 +439,7 @@ static cudaGraphExec_t run_graph(de_ctx* c, int32_t generations) {
   auto it = c->graphs.find(generations);
   if (it != c->graphs.end()) return it->second;
   ResidentShape shape;
-  const bool resident = resident_ready(c, &shape);
+  const bool resident = resident_ready(c, &shape), segments = c->batch && batch_seg_ready(c, generations);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return nullptr;
@@ -455,6 +455,8 @@ static cudaGraphExec_t run_graph(de_ctx* c, int32_t generations) {
       rp.gens = std::min(left, kResMaxGens);
       le = launch_resident(c->xo, c->obj, c->vidx, shape, rp, c->stream);
     }
+  } else if (segments) {
+    for (int32_t k = -1; k < generations && le == cudaSuccess; ++k) le = batch_seg_launch(c, k);
   } else {
     for (int32_t k = 0; k < generations && le == cudaSuccess; ++k) le = launch_generation(c, c->p);
   }

@@ -192,6 +192,70 @@ cudaError_t batch_launch_generation(de_ctx* c, bool, int) {
                                  c->batch_grid, c->stream);
 }
 
+// Segment runs pay from the second generation (128 instances, Cr = 0.9, us per
+// generation in runs of 2, 4, 100: 314, 236, 164 against 568, 554, 559) and while
+// 1 / (1 - Cr) <= 60 genes (Cr = 0.95 252 / 572, 0.97 362 / 589, 0.98 462 / 627;
+// longer segments come near to every slot) or rows have at most 8 slots. A batch
+// whose wait limit was set keeps the kernel with the wait.
+bool batch_seg_ready(de_ctx* c, int generations) {
+  if (generations < 2 || c->wait_ns != 0ull) return false;
+  int ns = 1;
+  for (int k = 0; k < c->n_inst; ++k) {
+    const int D4 = c->bp[k].D4;
+    if (c->bxo[k] == DE_XOVER_BIN || c->bgroup[k] > 32 || D4 > kStageMaxD4) return false;
+    if (D4 > 8 && (1.0 - c->bcr[k]) * 60.0 < 1.0) return false;
+    ns = std::max(ns, c->bobj[k] == DE_OBJ_GRIEWANK ? 3 : (c->bobj[k] == DE_OBJ_ACKLEY ? 2 : 1));
+  }
+  if (c->bseg.spans) return true;
+  if (prepare_batch_seg() != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+  std::vector<BatchSpan> sp;
+  long long rows = 0;
+  // instances of one objective together: warps that run together share code
+  std::vector<int> order((size_t)c->n_inst);
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return c->bobj[a] < c->bobj[b]; });
+  for (int k : order) {
+    for (int r = 0; r < c->bp[k].N; r += kSpanRows) {
+      BatchSpan s{};
+      s.inst = k;
+      s.row0 = r;
+      s.rows = std::min(kSpanRows, c->bp[k].N - r);
+      s.plan0 = c->brow_base[k] + r;
+      sp.push_back(s);
+    }
+    rows += c->bp[k].N;
+  }
+  BatchSeg b{};
+  b.nspans = (int)sp.size();
+  b.stride = 32 * ns;
+  BatchSpan* spans = (BatchSpan*)ctx_alloc(c, sp.size() * sizeof(BatchSpan));
+  b.sums = (float*)ctx_alloc(c, (size_t)rows * b.stride * sizeof(float));
+  b.won = (ushort4*)ctx_alloc(c, (size_t)rows * sizeof(ushort4));
+  b.done = (unsigned*)ctx_alloc(c, sizeof(unsigned));
+  if (spans && b.sums && b.won && b.done &&
+      cudaMemcpyAsync(spans, sp.data(), sp.size() * sizeof(BatchSpan), cudaMemcpyHostToDevice, c->stream) ==
+          cudaSuccess &&
+      cudaMemsetAsync(b.done, 0, sizeof(unsigned), c->stream) == cudaSuccess && sync_stream(c) == DE_OK) {
+    b.spans = spans;
+    c->bseg = b;
+    return true;
+  }
+  cudaGetLastError();
+  for (void* q : {(void*)spans, (void*)b.sums, (void*)b.won, (void*)b.done})
+    if (q) ctx_free(c, q);
+  return false;
+}
+
+cudaError_t batch_seg_launch(de_ctx* c, int k) {
+  return k < 0 ? launch_batch_seg_init(c->d_insts, c->bseg, c->stream)
+               : launch_batch_seg(c->d_insts, c->bseg, c->d_states, c->n_inst, c->stream);
+}
+
 // Plan tiles: 256 consecutive rows of one instance, instances in order.
 static int build_plan_tiles(de_ctx* c) {
   std::vector<BatchTile> pt;

@@ -77,6 +77,7 @@ struct de_ctx {
   std::vector<long long> brow_base;
   de::DevState* d_states = nullptr;
   int nctiles = 0, batch_grid = 0, max_pitch = 0;
+  de::BatchSeg bseg{};                   // segment runs (made by the first one)
   // shifted-rotated objectives (sr_api.cu)
   bool rotated = false;
   de::SrParams sp{};
@@ -116,6 +117,10 @@ int batch_set_base(de_ctx* c, int base);
 // Batched contexts (batch_api.cu).
 cudaError_t batch_launch_generation(de_ctx* c, bool with_debug_of_inst, int inst);
 int batch_stats(de_ctx* c, de_stats_t* out);
+// Whether a run of this many generations goes through batch_seg.cu (its buffers
+// made on first use), and one launch of it: k = -1 starts the run.
+bool batch_seg_ready(de_ctx* c, int generations);
+cudaError_t batch_seg_launch(de_ctx* c, int k);
 // Shifted-rotated objectives (sr_api.cu).
 int sr_setup(de_ctx* c, const de_objparams* prm);
 cudaError_t sr_launch_generation(de_ctx* c, const GenParams& p);

@@ -165,6 +165,19 @@ cudaError_t launch_batch_flow_fused(const BatchInst* insts, const BatchSpan* spa
                                     const BatchTile* ptiles, int nptiles, RowPlan32* plans, DevState* states,
                                     int n_inst, unsigned* ctr, int grid, unsigned long long wait_ns,
                                     cudaStream_t s);
+// runs of a batch of segment crossovers that touch only what the segments
+// touch (batch_seg.cu): the start of a run, then one launch per generation
+struct BatchSeg {
+  const BatchSpan* spans;      // every row of every instance, up to 32 per span
+  int nspans;
+  float* sums;                 // per row: `stride` floats, 32 partial sums per sum of the objective
+  int stride;
+  ushort4* won;                // per row: the slots (a0, n0, n1) that its other buffer lacks
+  unsigned* done;              // CTAs finished, zero between launches
+};
+cudaError_t prepare_batch_seg();
+cudaError_t launch_batch_seg_init(const BatchInst* insts, const BatchSeg& b, cudaStream_t s);
+cudaError_t launch_batch_seg(const BatchInst* insts, const BatchSeg& b, DevState* states, int n_inst, cudaStream_t s);
 // the span row kernel alone, one per crossover (batch_span_*.cu)
 cudaError_t launch_batch_span_bin(const BatchInst*, const BatchSpan*, int, const RowPlan32*, unsigned*, int, int,
                                   cudaStream_t);
