@@ -444,8 +444,7 @@ __global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const 
   __shared__ const float* rowp_all[kLsGroups][kLsE];
   const float** rowp = rowp_all[g];
   const int lane = t & 31, warp = t >> 5;
-  const int tx = lane & 15;
-  const int ebase = warp * 4 + (lane >> 4) * 2;    // the lane's first entry in the tile
+  const int ebase = warp * 4;                      // the warp's first entry in the tile
   const long long gen = p.st->gen;
   const uint8_t* slot_in = p.slots + (size_t)(gen & 1) * p.N;
   const int nrows = (int)*sp.amb_count;
@@ -483,11 +482,9 @@ __global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const 
       if (s0 < KS) issue(s0);
       cp_async_commit();
     }
-    float acc[2][4];
+    float acc[4][2];
 #pragma unroll
-    for (int e = 0; e < 2; ++e)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[e][c] = 0.0f;
+    for (int e = 0; e < 4; ++e) acc[e][0] = acc[e][1] = 0.0f;
     for (int step = 0; step < KS; ++step) {
       cp_async_wait<kLsStages - 2>();
       ls_group_sync(g);                             // this stage landed; every lane is done with the
@@ -506,27 +503,37 @@ __global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const 
       }
       __syncwarp();                                 // a of the warp's entries, written by the warp
       const float* as = As + ebase;
-      const float* bs = Bs + st * kLsK * kLsLdB + 4 * tx;
+      const float* bs = Bs + st * kLsK * kLsLdB + 2 * lane;
 #pragma unroll
       for (int k = 0; k < kLsK; ++k) {
-        const float2 av = *reinterpret_cast<const float2*>(as + k * kLsLdA);
-        const float4 bv = *reinterpret_cast<const float4*>(bs + k * kLsLdB);
+        const float4 av = *reinterpret_cast<const float4*>(as + k * kLsLdA);
+        const float2 bv = *reinterpret_cast<const float2*>(bs + k * kLsLdB);
         acc[0][0] = fmaf(av.x, bv.x, acc[0][0]);
         acc[0][1] = fmaf(av.x, bv.y, acc[0][1]);
-        acc[0][2] = fmaf(av.x, bv.z, acc[0][2]);
-        acc[0][3] = fmaf(av.x, bv.w, acc[0][3]);
         acc[1][0] = fmaf(av.y, bv.x, acc[1][0]);
         acc[1][1] = fmaf(av.y, bv.y, acc[1][1]);
-        acc[1][2] = fmaf(av.y, bv.z, acc[1][2]);
-        acc[1][3] = fmaf(av.y, bv.w, acc[1][3]);
+        acc[2][0] = fmaf(av.z, bv.x, acc[2][0]);
+        acc[2][1] = fmaf(av.z, bv.y, acc[2][1]);
+        acc[3][0] = fmaf(av.w, bv.x, acc[3][0]);
+        acc[3][1] = fmaf(av.w, bv.y, acc[3][1]);
       }
     }                                               // (the next step's group barrier orders the As reuse)
     cp_async_wait<0>();
+    // the layout of the tile reduction: lane tx of each half has the columns 4 tx
+    // .. 4 tx + 3, the lower half of one entry and the upper half of the next
+    const int tx = lane & 15;
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int ent = r0 + ebase + e;
+    for (int e = 0; e < 4; e += 2) {
+      float z[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float a = __shfl_sync(0xFFFFFFFFu, acc[e][c & 1], 2 * tx + (c >> 1));
+        const float b = __shfl_sync(0xFFFFFFFFu, acc[e + 1][c & 1], 2 * tx + (c >> 1));
+        z[c] = lane < 16 ? a : b;
+      }
+      const int ent = r0 + ebase + e + (lane >> 4);
       float sg, sw;
-      sr_tile_reduce(sp, acc[e], n0 + 4 * tx, sg, sw);
+      sr_tile_reduce(sp, z, n0 + 4 * tx, sg, sw);
       if (tx == 0 && ent < nrows) {
         sp.part2_g[(size_t)ent * sp.nct2 + ct] = sg;
         sp.part2_w[(size_t)ent * sp.nct2 + ct] = sw;
