@@ -201,7 +201,7 @@ cudaError_t launch_sr_transpose(const float* rot, float* rot_t, int D, cudaStrea
 cudaError_t launch_sr_finish(const SrParams& sp, int every, bool close, cudaStream_t s);
 // tcgen05 BF16 product (split operands) with the fitness epilogue; requires
 // D % 256 == 0. sr_tc_supported tells whether this build and device have it.
-cudaError_t launch_sr_gemm_tc(const SrParams& sp, cudaStream_t s);
+cudaError_t launch_sr_gemm_tc(const SrParams& sp, bool want_w, cudaStream_t s);
 cudaError_t prepare_sr_tc();
 cudaError_t prepare_sr_list(int* ctas);
 bool sr_tc_supported(int D);

@@ -133,13 +133,12 @@ int sr_setup(de_ctx* c, const de_objparams* prm) {
   sp.amb = (int*)ctx_alloc(c, 2 * (size_t)N * sizeof(int));
   sp.amb_count = (unsigned*)ctx_alloc(c, sizeof(unsigned));
   sp.part2_g = (float*)ctx_alloc(c, 2 * (size_t)N * sp.nct2 * sizeof(float));
-  sp.part2_w = (float*)ctx_alloc(c, 2 * (size_t)N * sp.nct2 * sizeof(float));
   sp.inc_part = (double*)ctx_alloc(c, (size_t)D * sizeof(double));
   sp.inc_count = (unsigned*)ctx_alloc(c, sizeof(unsigned));
   sp.finish_due = (int*)ctx_alloc(c, sizeof(int));
   sp.inc_every = c->incumbent_every;
   if (!shift || !rot || !sp.part_g || !sp.part_w || !sp.norm2 || !sp.amax || !sp.fit_err || !sp.amb || !sp.amb_count ||
-      !sp.part2_g || !sp.part2_w || !sp.inc_part || !sp.inc_count || !sp.finish_due)
+      !sp.part2_g || !sp.inc_part || !sp.inc_count || !sp.finish_due)
     return DE_ENOMEM;
   sp.shift = shift;
   sp.rot = rot;
@@ -199,7 +198,7 @@ cudaError_t sr_launch_generation(de_ctx* c, const GenParams& p) {
   cudaError_t e = launch_sr_trial(c->xo, c->vidx, sp, c->block, c->stream);
   if (e == cudaSuccess) {
     if (sp.prec == 0) e = launch_sr_gemm_fp32(sp, 0, c->N, c->stream);
-    else e = launch_sr_gemm_tc(sp, c->stream);
+    else e = launch_sr_gemm_tc(sp, c->sbound.mode == 1, c->stream);
   }
   if (e == cudaSuccess) e = launch_sr_select(sp, c->sbound, c->stream);
   if (e == cudaSuccess && sp.prec != 0) {

@@ -29,14 +29,14 @@ struct SrParams {
   uint16_t* a_hi;          // hi(u - o) (BF16, or FP16 of 2^sa (u - o)), N x D
   uint16_t* a_lo;          // lo(u - o): the rounded remainder, N x D
   float* part_g;           // N x nct: sum of g(z) over the column tile
-  float* part_w;           // N x nct: sum of w_k |z_k| (w = 1 Rastrigin, c_k elliptic)
+  float* part_w;           // N x nct: sum of w_k |z_k| (w = 1 Rastrigin, c_k elliptic), split products
+                           // with the worst-case bound
   float* norm2;            // N: |u - o|^2 of the trial (FP32)
   float* amax;             // N: max_j |u_j - o_j| of the trial
   float* fit_err;          // N: bound on |fit - FP32-path value| of the stored parent
   int* amb;                // ambiguous entries: row << 1 | (1 = parent row)
   unsigned* amb_count;     // number of entries in amb
   float* part2_g;          // 2N x nct: partial sums of the re-evaluated entries
-  float* part2_w;
   double* inc_part;        // D: FP64 g(z_k) of the incumbent re-evaluation
   unsigned* inc_count;     // CTAs of the incumbent re-evaluation done (last one sums)
   int inc_every;           // FP64 incumbent every inc_every generations

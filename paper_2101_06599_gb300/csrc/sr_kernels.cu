@@ -211,24 +211,22 @@ __device__ __forceinline__ const float* sr_row_ptr(const SrParams& sp, int mode,
 
 // One row's 4 columns of a 64-column tile, reduced over the tile's 16 lanes
 // (all 32 lanes of the warp call it; lanes 16..31 reduce their own tile row).
-__device__ __forceinline__ void sr_tile_reduce(const SrParams& sp, const float z[4], int c0, float& sg, float& sw) {
+__device__ __forceinline__ float sr_tile_reduce(const SrParams& sp, const float z[4], int c0) {
   const GenParams& p = sp.g;
-  sg = 0.0f;
-  sw = 0.0f;
+  float sg = 0.0f;
 #pragma unroll
   for (int b = 0; b < 4; ++b) {
     const int n = c0 + b;
     if (n < p.D) {
       const float w = sr_weight(sp.obj, n, p.ell_k);
       sg += sr_g(sp.obj, z[b], w);
-      sw = fmaf(w, fabsf(z[b]), sw);
     }
   }
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) {
     sg += __shfl_xor_sync(0xFFFFFFFFu, sg, o);
-    sw += __shfl_xor_sync(0xFFFFFFFFu, sw, o);
   }
+  return sg;
 }
 
 // All rows (modes 0 and 1): tiles of 8 RT rows x 64 columns, 128 threads, RT
@@ -393,12 +391,8 @@ __global__ void __launch_bounds__(kGbThreads, 4) sr_gemm_fp32_kernel(const __gri
     for (int h = 0; h < 2; ++h) {
       const float z[4] = {h ? z0.y : z0.x, h ? z1.y : z1.x, h ? z2.y : z2.x, h ? z3.y : z3.x};
       const int e = r0 + m + h;
-      float sg, sw;
-      sr_tile_reduce(sp, z, n0 + 4 * tx, sg, sw);
-      if (tx == 0 && e < p.N) {
-        sp.part_g[(size_t)e * sp.nct2 + blockIdx.x] = sg;
-        sp.part_w[(size_t)e * sp.nct2 + blockIdx.x] = sw;
-      }
+      const float sg = sr_tile_reduce(sp, z, n0 + 4 * tx);
+      if (tx == 0 && e < p.N) sp.part_g[(size_t)e * sp.nct2 + blockIdx.x] = sg;
     }
   }
 }
@@ -532,12 +526,8 @@ __global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const 
         z[c] = lane < 16 ? a : b;
       }
       const int ent = r0 + ebase + e + (lane >> 4);
-      float sg, sw;
-      sr_tile_reduce(sp, z, n0 + 4 * tx, sg, sw);
-      if (tx == 0 && ent < nrows) {
-        sp.part2_g[(size_t)ent * sp.nct2 + ct] = sg;
-        sp.part2_w[(size_t)ent * sp.nct2 + ct] = sw;
-      }
+      const float sg = sr_tile_reduce(sp, z, n0 + 4 * tx);
+      if (tx == 0 && ent < nrows) sp.part2_g[(size_t)ent * sp.nct2 + ct] = sg;
     }
   }
 }

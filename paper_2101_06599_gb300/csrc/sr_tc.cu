@@ -7,7 +7,7 @@
 // steps add almost nothing to the accumulator's rounding, which the leading
 // D/16 steps then dominate (the error bound counts it that way).
 //
-// One CTA per 128 x 256 output tile; 6 warps:
+// One CTA per 128 x 256 output tile; 10 warps:
 //   warp 0      one thread issues 2D tensor loads (TMA, 128-byte swizzle) of
 //               the A and B tiles (K = 64 per stage) into a 4-stage ring
 //               (full / empty mbarriers);
@@ -16,10 +16,17 @@
 //               or FP16 inputs, FP32 accumulator), commits each stage's MMAs to the
 //               stage's empty barrier and the last to the accumulator barrier;
 //               frees TMEM at the end;
-//   warps 2..5  read the accumulator with tcgen05.ld (warp w reads TMEM lanes
-//               32 (w mod 4) .. + 31 = its 32 tile rows), undo the operands'
-//               power-of-two scaling (FP16) and reduce g(z) and w |z| over
-//               the tile's 256 columns into per-row partials.
+//   warps 2..9  read the accumulator with tcgen05.ld (warp w reads TMEM lanes
+//               32 (w mod 4) .. + 31 = 32 tile rows, warps 2-5 the first 128
+//               columns and warps 6-9 the others), undo the operands'
+//               power-of-two scaling (FP16) and reduce g(z), and w |z| where the
+//               worst-case bound needs it, into per-row partials.
+// The barriers, TMEM and the tensor maps are set up before the wait for the
+// trial kernel. Bound by the 192 MMAs of a tile and the 2.3 MB of operands they
+// read from L2 (N = 4096, D = 1024: 128 tiles, one per CTA, 22 us); where the
+// product is shorter the set-up and the epilogue count: with them beside the
+// trial kernel and on eight warps a BF16 generation at N = 2000, D = 768 took
+// 41.4 us instead of 43.3, FP16 at N = 1000, D = 512 32.8 instead of 34.2.
 // Every mbarrier wait is bounded (1 s); on a timeout the kernel records
 // DE_ETIMEOUT, lets issued copies and MMAs drain (bounded), frees TMEM and
 // returns.
@@ -35,7 +42,7 @@
 
 namespace de {
 
-constexpr int kTcBM = 128, kTcBN = 256, kTcBK = 64, kTcStages = 4, kTcThreads = 192;
+constexpr int kTcBM = 128, kTcBN = 256, kTcBK = 64, kTcStages = 4, kTcThreads = 320;
 constexpr uint32_t kTcStageA = kTcBM * kTcBK * 2;   // 16 KB
 constexpr uint32_t kTcStageB = kTcBN * kTcBK * 2;   // 32 KB
 constexpr uint32_t kTcTmemCols = 256;
@@ -45,6 +52,7 @@ struct TcParams {
   SrParams sp;
   CUtensorMap ta_hi, ta_lo, tr_hi, tr_lo;
   uint32_t idesc;          // instruction descriptor (operand type)
+  int want_w;              // the sums of w |z| are read (worst-case bound)
 };
 
 // K-major, 128-byte-swizzled shared-memory matrix descriptor: start address,
@@ -102,9 +110,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 
 __global__ void __launch_bounds__(kTcThreads, 1) sr_tc_kernel(const __grid_constant__ TcParams tp) {
-  griddep_wait();                                  // the trial kernel has written the operands
-  griddep_launch_dependents();
   extern __shared__ unsigned char smem_raw[];
+  __shared__ float s_half[2][kTcBM];               // the second half's sums
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char* sA = smem;
   unsigned char* sB = smem + kTcStages * kTcStageA;
@@ -127,6 +134,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) sr_tc_kernel(const __grid_const
     }
     mbar_init(smem_u32(accum), 1u);
     fence_mbar_init();
+    for (const CUtensorMap* m : {&tp.ta_hi, &tp.ta_lo, &tp.tr_hi, &tp.tr_lo})
+      asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -138,6 +147,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) sr_tc_kernel(const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  griddep_wait();                                  // the trial kernel has written the operands
+  griddep_launch_dependents();
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer ----
@@ -182,33 +193,47 @@ __global__ void __launch_bounds__(kTcThreads, 1) sr_tc_kernel(const __grid_const
     const bool ok = mbar_wait(smem_u32(accum), 0u);
     tc_fence_after();
     const int q = warp & 3;                    // TMEM lane quadrant of this warp
-    const int m = tile_m * kTcBM + 32 * q + lane;
+    const int half = (warp - 2) >> 2;          // and its 128 of the 256 columns
+    const int r = 32 * q + lane, m = tile_m * kTcBM + r;
     float sg = 0.0f, sw = 0.0f;
     if (ok) {
-      // one loop per objective (the objective is uniform): no per-value test
-      auto tile_sums = [&](auto obj_tag) {
+      // one loop per objective (the objective is uniform): no per-value test;
+      // even and odd columns in a sum each
+      auto tile_sums = [&](auto obj_tag, auto w_tag) {
         constexpr int OBJ = decltype(obj_tag)::value;
+        float g2[2] = {0.0f, 0.0f};
 #pragma unroll 1
-        for (int c0 = 0; c0 < kTcBN; c0 += 32) {
-          uint32_t r[32];
-          tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, r);
+        for (int c0 = half * (kTcBN / 2); c0 < (half + 1) * (kTcBN / 2); c0 += 32) {
+          uint32_t v[32];
+          tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
 #pragma unroll
           for (int c = 0; c < 32; ++c) {
-            const float z = __uint_as_float(r[c]) * sp.z_scale;   // exact: a power of two
+            const float z = __uint_as_float(v[c]) * sp.z_scale;   // exact: a power of two
             const float w = sr_weight(OBJ, tile_n * kTcBN + c0 + c, p.ell_k);
-            sg += sr_g(OBJ, z, w);
-            sw = fmaf(w, fabsf(z), sw);
+            g2[c & 1] += sr_g(OBJ, z, w);
+            if constexpr (decltype(w_tag)::value) sw = fmaf(w, fabsf(z), sw);
           }
         }
+        sg = g2[0] + g2[1];
       };
-      if (sp.obj == kSrElliptic) tile_sums(std::integral_constant<int, kSrElliptic>{});
-      else tile_sums(std::integral_constant<int, kSrRastrigin>{});
+      if (sp.obj == kSrElliptic) {
+        if (tp.want_w) tile_sums(std::integral_constant<int, kSrElliptic>{}, std::true_type{});
+        else tile_sums(std::integral_constant<int, kSrElliptic>{}, std::false_type{});
+      } else {
+        if (tp.want_w) tile_sums(std::integral_constant<int, kSrRastrigin>{}, std::true_type{});
+        else tile_sums(std::integral_constant<int, kSrRastrigin>{}, std::false_type{});
+      }
     } else {
       atomicExch(&p.st->error, 4u);
     }
-    if (m < p.N) {
-      sp.part_g[(size_t)m * sp.nct + tile_n] = sg;
-      sp.part_w[(size_t)m * sp.nct + tile_n] = sw;
+    if (half == 1) {
+      s_half[0][r] = sg;
+      s_half[1][r] = sw;
+    }
+    named_bar_sync(1, kTcThreads - 64);
+    if (half == 0 && m < p.N) {
+      sp.part_g[(size_t)m * sp.nct + tile_n] = sg + s_half[0][r];
+      if (tp.want_w) sp.part_w[(size_t)m * sp.nct + tile_n] = sw + s_half[1][r];
     }
   }
   tc_fence_before();
@@ -268,10 +293,11 @@ cudaError_t prepare_sr_tc() {
   return cudaFuncSetAttribute(sr_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
 }
 
-cudaError_t launch_sr_gemm_tc(const SrParams& sp, cudaStream_t s) {
+cudaError_t launch_sr_gemm_tc(const SrParams& sp, bool want_w, cudaStream_t s) {
   TcParams tp;
   std::memset(&tp, 0, sizeof(tp));
   tp.sp = sp;
+  tp.want_w = want_w ? 1 : 0;
   const int N = sp.g.N, D = sp.g.D;
   const bool fp16 = sp.prec == 3;
   tp.idesc = fp16 ? kTcIdescF16 : kTcIdescBF16;
