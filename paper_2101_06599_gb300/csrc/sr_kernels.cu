@@ -565,9 +565,25 @@ cudaError_t launch_sr_transpose(const float* rot, float* rot_t, int D, cudaStrea
 // ---------------------------------------------------------------------------
 // decisions
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float sr_row_value(const float* pg, int nct) {
-  float f = 0.0f;
-  for (int c = 0; c < nct; ++c) f += pg[c];
+// The partials of a row are loaded 16 at a time before they are added in order: a
+// load per addition was a round trip to L2 per tile in one dependent row (D /
+// 256 in the selection, D / 64 twice in the resolution). tsq, if wanted: the sum
+// of their squares.
+template <bool kSquares = false>
+__device__ __forceinline__ float sr_row_value(const float* pg, int nct, float* tsq = nullptr) {
+  float f = 0.0f, s = 0.0f;
+  for (int c0 = 0; c0 < nct; c0 += 16) {
+    float v[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) v[c] = (c0 + c < nct) ? pg[c0 + c] : 0.0f;
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+      if (c0 + c < nct) {
+        f += v[c];
+        if constexpr (kSquares) s = fmaf(v[c], v[c], s);
+      }
+  }
+  if constexpr (kSquares) *tsq = s;
   return (f != f) ? __int_as_float(0x7F800000) : f;
 }
 
@@ -646,20 +662,17 @@ __global__ void sr_select_kernel(const __grid_constant__ SrParams sp, SrBound bn
   float f = 0.0f, bx = 0.0f;
   if (i < p.N) {
     const int si = slot_in[i];
-    f = sr_row_value(sp.part_g + (size_t)i * sp.nct, sp.nct);
-    float bu = 0.0f;
-    if (sp.prec != 0) {
-      float sw = 0.0f, tsq = 0.0f;                 // sum of the tile partials' squares
-      for (int c = 0; c < sp.nct; ++c) {
-        const float t = sp.part_g[(size_t)i * sp.nct + c];
-        tsq = fmaf(t, t, tsq);
-      }
-      if (bnd.mode == 1)
-        for (int c = 0; c < sp.nct; ++c) sw += sp.part_w[(size_t)i * sp.nct + c];
-      bu = sr_bound(sp.obj, sp.norm2[i], sp.amax[i], sw, f, tsq * 1.0001f, p.D, bnd);
-    }
     const float fx = p.fit[i];
     bx = sp.fit_err[i];
+    const float norm2 = sp.norm2[i], amax = sp.amax[i];
+    float bu = 0.0f, tsq;                          // sum of the tile partials' squares
+    f = sr_row_value<true>(sp.part_g + (size_t)i * sp.nct, sp.nct, &tsq);
+    if (sp.prec != 0) {
+      float sw = 0.0f;
+      if (bnd.mode == 1)
+        for (int c = 0; c < sp.nct; ++c) sw += sp.part_w[(size_t)i * sp.nct + c];
+      bu = sr_bound(sp.obj, norm2, amax, sw, f, tsq * 1.0001f, p.D, bnd);
+    }
     if (bu == 0.0f && bx == 0.0f) decision = (f < fx) ? 1 : 0;
     else if (f + bu < fx - bx) decision = 1;
     else if (f - bu >= fx + bx) decision = 0;
@@ -718,15 +731,16 @@ __global__ void sr_resolve_kernel(const __grid_constant__ SrParams sp) {
   int i = 0;
   if (e < n && !(sp.amb[e] & 1)) {                 // parents are read by their trial's entry
     i = sp.amb[e] >> 1;
+    const int si = slot_in[i];
+    const float fp = p.fit[i];
+    const bool parent = e + 1 < n && sp.amb[e + 1] == ((i << 1) | 1);
     fu = sr_row_value(sp.part2_g + (size_t)e * sp.nct2, sp.nct2);
-    float fx = p.fit[i];
-    if (e + 1 < n && sp.amb[e + 1] == ((i << 1) | 1)) {
-      fx = sr_row_value(sp.part2_g + (size_t)(e + 1) * sp.nct2, sp.nct2);
-      p.fit[i] = fx;                               // the parent's exact FP32-path value
+    const float fe = parent ? sr_row_value(sp.part2_g + (size_t)(e + 1) * sp.nct2, sp.nct2) : fp;
+    if (parent) {
+      p.fit[i] = fe;                               // the parent's exact FP32-path value
       sp.fit_err[i] = 0.0f;
     }
-    const int si = slot_in[i];
-    acc = fu < fx;
+    acc = fu < fe;
     if (acc) {
       slot_out[i] = (uint8_t)(1 - si);
       p.fit[i] = fu;
