@@ -398,57 +398,73 @@ __global__ void __launch_bounds__(kGbThreads, 4) sr_gemm_fp32_kernel(const __gri
 }
 
 // The ambiguous entries (mode 2; split-operand paths only, so D % 256 == 0):
-// work items of 16 entries x 64 columns, taken by groups of 4 warps (2
-// entries x 4 columns per lane: lanes 0-15 take entries 0-1 of the warp, lanes
-// 16-31 entries 2-3, and lane tx = lane & 15 columns 4 tx .. 4 tx + 3 of the
-// 64-column tile, the layout the tile reduction expects). Each group has its
-// own 4-stage cp.async ring of 64-deep slices of the entries' rows of x, o
-// and rows of R^T (three stages in flight cover the L2 latency of the short
-// per-stage work) and its own named barrier. Once a stage has landed, each
-// warp forms a = fl(x - o) K-major for its own four entries (so only a warp
-// barrier follows), and the inner loop is an 8-byte and a 16-byte shared load
-// and eight FMAs per k: every z stays one FMA chain over j ascending. The list is
-// short (a few hundred entries) and each chain is D FMAs long, so the time is
-// set by the busiest SM. Two groups per CTA and a ring per group that needs
-// more than half an SM's shared memory for the pair put exactly one CTA on
-// each SM; the grid is one CTA per SM, group g of CTA b takes items
-// b + g * grid, b + (2 + g) * grid, ..., so the first items of a short list
-// land on distinct SMs whatever order the CTAs are placed in.
-constexpr int kLsE = 16, kLsN = 64, kLsK = 64, kLsStages = 4, kLsGroupThreads = 128, kLsGroups = 2;
+// work items of 4 WE entries x 64 columns, taken by groups of 4 warps: a warp has
+// WE entries (WE = 2, 4 or 8), a lane the columns 2 lane and 2 lane + 1 of the
+// tile for all of them, so a k costs a broadcast of the entries' a, 8 bytes of R^T
+// per lane and 2 WE FMAs. Each group has its own 3-stage cp.async ring of 64-deep
+// slices of the entries' rows of x, o and rows of R^T and its own named barrier.
+// Once a stage has landed, each warp forms a = fl(x - o) K-major for its own
+// entries (so only a warp barrier follows): every z stays one FMA chain over j
+// ascending. The list is short (a few hundred entries) and each chain is D FMAs
+// long, so the time is set by the busiest SM, and there by the latency of a warp's
+// step: about 27, 37 and 52 cycles per k for WE = 2, 4 and 8, one warp per
+// scheduler (ls_warp_entries has the rule). Generations by WE = 2, 4, 8, us: 71 rows
+// (FP16 Rastrigin, N = 4096, D = 1024) 63.4, 59.2, 62.2 and 58.3 by the rule, which
+// follows each list; 141 rows (BF16) 86.3, 71.2, 73.2 and 70.3; 9 rows (N = 1000, D
+// = 512) 29.9, 31.7, 36.3; 563 rows (N = 16384) 300, 237, 210. Two groups per CTA and a ring per
+// group that needs more than half an SM's shared memory for the pair put exactly
+// one CTA on each SM; the grid is one CTA per SM, group g of CTA b takes items b +
+// g * grid, b + (2 + g) * grid, ..., so the first items of a short list land on
+// distinct SMs whatever order the CTAs are placed in.
+constexpr int kLsMaxE = 32, kLsN = 64, kLsK = 64, kLsStages = 3, kLsGroupThreads = 128, kLsGroups = 2;
 constexpr int kLsThreads = kLsGroups * kLsGroupThreads;
-constexpr int kLsLdX = kLsK + 4, kLsLdB = kLsN + 4, kLsLdA = kLsE + 4;   // floats per row
-constexpr int kLsGroupFloats = kLsStages * (kLsE * kLsLdX + kLsK + kLsK * kLsLdB) + kLsK * kLsLdA;
+constexpr int kLsLdX = kLsK + 4, kLsLdB = kLsN + 4;   // floats per row
+constexpr int kLsGroupFloats = kLsStages * (kLsMaxE * kLsLdX + kLsK + kLsK * kLsLdB) + kLsK * (kLsMaxE + 4);
 constexpr size_t kLsSmem = sizeof(float) * (size_t)kLsGroups * kLsGroupFloats;
 static_assert(kLsSmem > 114 * 1024 && kLsSmem <= 227 * 1024, "one CTA per SM");
+
+// Entries per warp for a list of n entries and ct column tiles on `grid` CTAs:
+// the least estimated time: a round of items (one group per SM) at the cost above,
+// two rounds side by side 1.6 of it.
+__device__ __forceinline__ int ls_warp_entries(int n, int ct, int grid) {
+  int best = 8;
+  float cost = 1e30f;
+  const float per_k[3] = {27.0f, 37.0f, 52.0f};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int we = 2 << c, items = (n + 4 * we - 1) / (4 * we) * ct, rounds = (items + grid - 1) / grid;
+    const float t = per_k[c] * (1.6f * (float)(rounds / 2) + (float)(rounds % 2));
+    if (t < cost) {
+      cost = t;
+      best = we;
+    }
+  }
+  return best;
+}
 
 __device__ __forceinline__ void ls_group_sync(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "n"(kLsGroupThreads) : "memory");
 }
 
-__global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const __grid_constant__ SrParams sp) {
-  griddep_wait();                                  // the previous kernel of the generation is done
-  griddep_launch_dependents();
+template <int WE>
+__device__ __forceinline__ void ls_items(const SrParams& sp, float* ls_smem, const float** rowp, int nrows) {
+  constexpr int kLsE = 4 * WE, kLsLdA = kLsE + 4;
   const GenParams& p = sp.g;
-  extern __shared__ __align__(16) float ls_smem[];
   const int g = threadIdx.x / kLsGroupThreads, t = threadIdx.x % kLsGroupThreads;
   float* Xs = ls_smem + (size_t)g * kLsGroupFloats;  // [stage][entry][kLsLdX]: raw x
   float* Os = Xs + kLsStages * kLsE * kLsLdX;      // [stage][k]: o
   float* Bs = Os + kLsStages * kLsK;               // [stage][k][kLsLdB]: R^T rows
   float* As = Bs + kLsStages * kLsK * kLsLdB;      // [k][kLsLdA]: a per entry
-  __shared__ const float* rowp_all[kLsGroups][kLsE];
-  const float** rowp = rowp_all[g];
   const int lane = t & 31, warp = t >> 5;
-  const int ebase = warp * 4;                      // the warp's first entry in the tile
+  const int ebase = warp * WE;               // the warp's first entry in the tile
   const long long gen = p.st->gen;
   const uint8_t* slot_in = p.slots + (size_t)(gen & 1) * p.N;
-  const int nrows = (int)*sp.amb_count;
   const int KS = p.D / kLsK, ctiles = p.D / kLsN;
   const int items = ((nrows + kLsE - 1) / kLsE) * ctiles;
   int n0 = 0;
 
-  // one stage: x 16 entries x 16 chunks of 16 bytes (two per thread), o 16
-  // chunks, R^T 64 rows x 16 chunks (8 per thread); entries past the list
-  // read zeros
+  // one stage: x 4 WE entries x 16 chunks of 16 bytes, o 16 chunks, R^T 64 rows x
+  // 16 chunks (8 per thread); entries past the list read zeros
   auto issue = [&](int step) {
     const int st = step % kLsStages, k0 = step * kLsK;
 #pragma unroll
@@ -476,9 +492,9 @@ __global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const 
       if (s0 < KS) issue(s0);
       cp_async_commit();
     }
-    float acc[4][2];
+    float acc[WE][2];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) acc[e][0] = acc[e][1] = 0.0f;
+    for (int e = 0; e < WE; ++e) acc[e][0] = acc[e][1] = 0.0f;
     for (int step = 0; step < KS; ++step) {
       cp_async_wait<kLsStages - 2>();
       ls_group_sync(g);                             // this stage landed; every lane is done with the
@@ -488,28 +504,35 @@ __global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const 
       const int st = step % kLsStages;
 #pragma unroll
       for (int kk = lane; kk < kLsK; kk += 32) {   // a = fl(x - o): k = kk, the warp's 4 entries
-        const int m0 = warp * 4;
-        const float* xs = Xs + (st * kLsE + m0) * kLsLdX + kk;
+        const float* xs = Xs + (st * kLsE + ebase) * kLsLdX + kk;
         const float o = Os[st * kLsK + kk];
-        *reinterpret_cast<float4*>(As + kk * kLsLdA + m0) =
-            make_float4(__fsub_rn(xs[0], o), __fsub_rn(xs[kLsLdX], o), __fsub_rn(xs[2 * kLsLdX], o),
-                        __fsub_rn(xs[3 * kLsLdX], o));
+#pragma unroll
+        for (int e = 0; e < WE; e += 2)
+          *reinterpret_cast<float2*>(As + kk * kLsLdA + ebase + e) =
+              make_float2(__fsub_rn(xs[e * kLsLdX], o), __fsub_rn(xs[(e + 1) * kLsLdX], o));
       }
       __syncwarp();                                 // a of the warp's entries, written by the warp
       const float* as = As + ebase;
       const float* bs = Bs + st * kLsK * kLsLdB + 2 * lane;
 #pragma unroll
       for (int k = 0; k < kLsK; ++k) {
-        const float4 av = *reinterpret_cast<const float4*>(as + k * kLsLdA);
         const float2 bv = *reinterpret_cast<const float2*>(bs + k * kLsLdB);
-        acc[0][0] = fmaf(av.x, bv.x, acc[0][0]);
-        acc[0][1] = fmaf(av.x, bv.y, acc[0][1]);
-        acc[1][0] = fmaf(av.y, bv.x, acc[1][0]);
-        acc[1][1] = fmaf(av.y, bv.y, acc[1][1]);
-        acc[2][0] = fmaf(av.z, bv.x, acc[2][0]);
-        acc[2][1] = fmaf(av.z, bv.y, acc[2][1]);
-        acc[3][0] = fmaf(av.w, bv.x, acc[3][0]);
-        acc[3][1] = fmaf(av.w, bv.y, acc[3][1]);
+        float av[WE];
+        if constexpr (WE == 2) {
+          const float2 a = *reinterpret_cast<const float2*>(as + k * kLsLdA);
+          av[0] = a.x; av[1] = a.y;
+        } else {
+#pragma unroll
+          for (int e = 0; e < WE; e += 4) {
+            const float4 a = *reinterpret_cast<const float4*>(as + k * kLsLdA + e);
+            av[e] = a.x; av[e + 1] = a.y; av[e + 2] = a.z; av[e + 3] = a.w;
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < WE; ++e) {
+          acc[e][0] = fmaf(av[e], bv.x, acc[e][0]);
+          acc[e][1] = fmaf(av[e], bv.y, acc[e][1]);
+        }
       }
     }                                               // (the next step's group barrier orders the As reuse)
     cp_async_wait<0>();
@@ -517,7 +540,7 @@ __global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const 
     // .. 4 tx + 3, the lower half of one entry and the upper half of the next
     const int tx = lane & 15;
 #pragma unroll
-    for (int e = 0; e < 4; e += 2) {
+    for (int e = 0; e < WE; e += 2) {
       float z[4];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -529,6 +552,20 @@ __global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const 
       const float sg = sr_tile_reduce(sp, z, n0 + 4 * tx);
       if (tx == 0 && ent < nrows) sp.part2_g[(size_t)ent * sp.nct2 + ct] = sg;
     }
+  }
+}
+
+__global__ void __launch_bounds__(kLsThreads, 1) sr_gemm_fp32_list_kernel(const __grid_constant__ SrParams sp) {
+  griddep_wait();                                  // the previous kernel of the generation is done
+  griddep_launch_dependents();
+  extern __shared__ __align__(16) float ls_smem[];
+  __shared__ const float* rowp[kLsGroups][kLsMaxE];
+  const float** mine = rowp[threadIdx.x / kLsGroupThreads];
+  const int nrows = (int)*sp.amb_count;
+  switch (ls_warp_entries(nrows, sp.g.D / kLsN, (int)gridDim.x)) {
+    case 2: ls_items<2>(sp, ls_smem, mine, nrows); break;
+    case 4: ls_items<4>(sp, ls_smem, mine, nrows); break;
+    default: ls_items<8>(sp, ls_smem, mine, nrows); break;
   }
 }
 
@@ -788,8 +825,8 @@ cudaError_t launch_sr_gemm_fp32(const SrParams& sp, int mode, int max_rows, cuda
   const unsigned gx = (unsigned)((sp.g.D + kGbN - 1) / kGbN);
   if (mode == 2) {                                // split-operand paths: D % 256 == 0
     if (sp.g.D % kLsN != 0) return cudaErrorInvalidValue;
-    const int items = ((max_rows + kLsE - 1) / kLsE) * (sp.g.D / kLsN);
-    const int grid = std::max(1, std::min(sp.list_ctas, (items + kLsGroups - 1) / kLsGroups));
+    const long long items = (long long)((max_rows + 7) / 8) * (sp.g.D / kLsN);   // of the smallest tiles
+    const int grid = (int)std::max(1LL, std::min((long long)sp.list_ctas, items));
     return launch_pdl(sr_gemm_fp32_list_kernel, dim3((unsigned)grid), dim3(kLsThreads), kLsSmem, s, sp);
   }
   // Rows per tile (8 RT): every SM works through ceil(tiles / SMs) of them, each
