@@ -405,7 +405,9 @@ static bool resident_ready(de_ctx* c, ResidentShape* shape) {
   if (c->p.base == kBaseBest) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-  const bool ok = prepare_resident(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR, c->sm_count,
+  shape->cluster = prepare_cluster(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR);
+  const bool ok = shape->cluster ||
+                  prepare_resident(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR, c->sm_count,
                                    c->smem_optin, shape);
   cudaGetLastError();
   if (!ok) return false;
@@ -453,7 +455,8 @@ static cudaGraphExec_t run_graph(de_ctx* c, int32_t generations) {
     rp.row_threads = c->block;
     for (int32_t left = generations; left > 0 && le == cudaSuccess; left -= rp.gens) {
       rp.gens = std::min(left, kResMaxGens);
-      le = launch_resident(c->xo, c->obj, c->vidx, shape, rp, c->stream);
+      le = shape.cluster ? launch_cluster(c->xo, c->obj, c->p, rp.gens, &c->res_state->hist, c->stream)
+                         : launch_resident(c->xo, c->obj, c->vidx, shape, rp, c->stream);
     }
   } else if (segments) {
     for (int32_t k = -1; k < generations && le == cudaSuccess; ++k) le = batch_seg_launch(c, k);

@@ -35,7 +35,7 @@ static int sums_of(int obj) {
 bool prepare_resident(int xo, int obj, int vidx, int block, int N, int D4, double CR, int sm_count, int smem_optin,
                       ResidentShape* out) {
   if (vidx > 1 || block > 256 || sm_count <= 0) return false;
-  ResidentShape s;
+  ResidentShape s{};
   s.rpc = (N + sm_count - 1) / sm_count;
   s.grid = (N + s.rpc - 1) / s.rpc;
   const int nw = block / 32;

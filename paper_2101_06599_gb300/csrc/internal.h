@@ -71,6 +71,7 @@ struct ResidentShape {
   int grid, block, rpc, groups;
   bool seg;                    // the kernel for segments
   size_t smem;
+  bool cluster;                // gen_cluster.cu instead (the rest then says nothing)
 };
 // The launch shape for rows of block x kVecChoices[vidx] slots, and the
 // kernel's attributes set for it; false if the population does
@@ -85,6 +86,11 @@ const void* resident_entry_ackley(bool seg, int vidx);
 const void* resident_entry_rosenbrock(bool seg, int vidx);
 const void* resident_entry_griewank(bool seg, int vidx);
 const void* resident_entry_elliptic(bool seg, int vidx);
+
+// The same for small populations, in one cluster (gen_cluster.cu). hist: the
+// ResState's, all ones between launches.
+bool prepare_cluster(int xo, int obj, int vidx, int block, int N, int D4, double CR);
+cudaError_t launch_cluster(int xo, int obj, const GenParams& p, int gens, unsigned long long* hist, cudaStream_t s);
 
 // Batched instances (batch_kernel.cu): one descriptor per instance and a
 // tile list; a tile is 256 / group rows of one instance.

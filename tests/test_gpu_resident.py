@@ -1,4 +1,5 @@
-"""Whole runs in one launch (gen_resident.cuh) against one launch per generation.
+"""Whole runs in one launch (gen_resident.cuh; gen_cluster.cu for up to 248 rows
+of D <= 128) against one launch per generation.
 
 de_run of a population that fits on the chip makes many generations in one
 launch; de_step, and de_run under de_set_kernel(1), launch each generation.
@@ -16,7 +17,7 @@ from paper_2101_06599_gb300 import workloads as W
 # edges: the smallest N, one row per CTA and several, a partial last CTA, more
 # than 32 rows per CTA (several barrier words), rows of one warp / one slot,
 # D % 4 != 0, two slots per thread, the longest rows of the kernel
-SHAPES = [(4, 1), (5, 3), (100, 30), (151, 127), (153, 128), (300, 500), (457, 1001), (1024, 1000), (301, 1029),
+SHAPES = [(4, 1), (5, 3), (8, 128), (9, 4), (100, 30), (151, 127), (153, 128), (248, 33), (249, 33), (300, 500), (457, 1001), (1024, 1000), (301, 1029),
           (160, 2047), (5000, 30), (4864, 129), (4865, 130), (9000, 61)]
 
 
@@ -71,6 +72,18 @@ def test_segments_that_wrap(obj, D):
         a, b = _pair(2500, D, F=0.7, CR=cr, xo="nec", obj=obj, bounds=W.BOXES[obj], seed=D)
         a.run(12)
         b.run(12)
+        _same(_state(a), _state(b))
+
+
+@pytest.mark.parametrize("xo,cr", [("nec", 0.97), ("exp", 0.4), ("bin", 0.6)])
+def test_one_cluster_edges(xo, cr):
+    """Rows and slots at the edges of the cluster's CTAs and of what it takes."""
+    for N, D in ((4, 2), (7, 31), (8, 4), (9, 5), (64, 127), (160, 128), (161, 65), (241, 64), (248, 61)):
+        obj = ("rosenbrock", "ackley", "griewank")[(N + D) % 3]
+        a, b = _pair(N, D, F=0.5, CR=cr, xo=xo, obj=obj, bounds=W.BOXES[obj], seed=N)
+        for count in (2, 9, 40):
+            a.run(count)
+            b.run(count)
         _same(_state(a), _state(b))
 
 
