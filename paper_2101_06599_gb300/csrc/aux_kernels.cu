@@ -217,6 +217,63 @@ __global__ void normalize_kernel(const __grid_constant__ GenParams p) {
   if (threadIdx.x == 0) sl[i] = 0;
 }
 
+// Dense rows of D genes in page-locked host memory: a thread takes 16 bytes of it
+// at a time, whatever rows they belong to, so that the link sees whole lines.
+__global__ void __launch_bounds__(256) rows_out_kernel(const __grid_constant__ GenParams p, float* __restrict__ pop,
+                                                       float* __restrict__ fit) {
+  const uint8_t* slots = p.slots + (size_t)(p.st->gen & 1) * p.N;
+  const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+  const size_t total = (size_t)p.N * p.D;
+  for (size_t e = 4 * t0; e < total; e += 4 * step) {
+    size_t i = e / p.D;
+    int j = (int)(e - i * p.D);
+    float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (e + k < total) lane_of(v, k) = ((slots[i] ? p.pop1 : p.pop0) + i * p.pitch)[j];
+      if (++j == p.D) {
+        j = 0;
+        ++i;
+      }
+    }
+    if (e + 4 <= total) {
+      *reinterpret_cast<float4*>(pop + e) = v;
+    } else {
+      for (int k = 0; e + k < total; ++k) pop[e + k] = lane_of(v, k);
+    }
+  }
+  if (fit)
+    for (size_t i = t0; i < (size_t)p.N; i += step) fit[i] = p.fit[i];
+}
+
+__global__ void __launch_bounds__(256) rows_in_kernel(const __grid_constant__ GenParams p, int parity,
+                                                      const float* __restrict__ pop, const float* __restrict__ fit) {
+  const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+  const size_t total = (size_t)p.N * p.D;
+  for (size_t e = 4 * t0; e < total; e += 4 * step) {
+    float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (e + 4 <= total) {
+      v = *reinterpret_cast<const float4*>(pop + e);
+    } else {
+      for (int k = 0; e + k < total; ++k) lane_of(v, k) = pop[e + k];
+    }
+    size_t i = e / p.D;
+    int j = (int)(e - i * p.D);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (e + k < total) p.pop0[i * p.pitch + j] = lane_of(v, k);
+      if (++j == p.D) {
+        j = 0;
+        ++i;
+      }
+    }
+  }
+  for (size_t i = t0; i < (size_t)p.N; i += step) {
+    p.slots[(size_t)parity * p.N + i] = 0;
+    if (fit) p.fit[i] = fit[i];
+  }
+}
+
 static unsigned grid_for(size_t work, unsigned block) {
   size_t g = (work + block - 1) / block;
   if (g > 152u * 32u) g = 152u * 32u;   // 152 SMs; grid-stride beyond that
@@ -245,6 +302,14 @@ cudaError_t launch_best_gather(const GenParams& p, void* staging, cudaStream_t s
 }
 cudaError_t launch_normalize(const GenParams& p, cudaStream_t s) {
   normalize_kernel<<<(unsigned)p.N, 128, 0, s>>>(p);
+  return cudaGetLastError();
+}
+cudaError_t launch_rows_out(const GenParams& p, float* pop, float* fit, cudaStream_t s) {
+  rows_out_kernel<<<grid_for(((size_t)p.N * p.D + 3) / 4, 256), 256, 0, s>>>(p, pop, fit);
+  return cudaGetLastError();
+}
+cudaError_t launch_rows_in(const GenParams& p, int parity, const float* pop, const float* fit, cudaStream_t s) {
+  rows_in_kernel<<<grid_for(((size_t)p.N * p.D + 3) / 4, 256), 256, 0, s>>>(p, parity, pop, fit);
   return cudaGetLastError();
 }
 

@@ -364,9 +364,8 @@ int de_batch_create(de_ctx** out, int32_t n_inst, const de_instance_spec* specs,
   }
   unsigned char* arena = (unsigned char*)ctx_alloc(c, bytes);
   c->d_insts = (BatchInst*)ctx_alloc(c, (size_t)n_inst * sizeof(BatchInst));
-  c->staging = ctx_alloc(c, kStagingHeader + (size_t)c->max_pitch * sizeof(float));
   c->host_pinned_bytes = std::max(kStagingHeader + (size_t)c->max_pitch * sizeof(float), sizeof(DevState));
-  if (!arena || !c->d_insts || !c->staging || cudaMallocHost(&c->host_pinned, c->host_pinned_bytes) != cudaSuccess) {
+  if (!arena || !c->d_insts || cudaMallocHost(&c->host_pinned, c->host_pinned_bytes) != cudaSuccess) {
     cudaGetLastError();
     de_destroy(c);
     return DE_ENOMEM;
@@ -461,11 +460,7 @@ int de_batch_best(de_ctx* c, int32_t inst, float* x_out, double* f_out, int32_t*
   if (!c || !c->batch) return c ? DE_ESTATE : DE_EINVAL;
   if (inst < 0 || inst >= c->n_inst) return DE_EINVAL;
   const GenParams& p = c->bp[inst];
-  cudaError_t e = launch_best_gather(p, c->staging, c->stream);
-  const size_t bytes = kStagingHeader + (size_t)p.D * sizeof(float);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(c->host_pinned, c->staging, bytes, cudaMemcpyDeviceToHost, c->stream);
-  if (e != cudaSuccess) return DE_ECUDA;
+  if (launch_best_gather(p, c->host_pinned, c->stream) != cudaSuccess) return DE_ECUDA;
   const int rc = sync_stream(c);
   if (rc != DE_OK) return rc;
   const unsigned char* h = static_cast<const unsigned char*>(c->host_pinned);
@@ -508,13 +503,7 @@ int de_batch_get_population(de_ctx* c, int32_t inst, float* pop_out, float* fit_
   if (!c->batch) return DE_ESTATE;
   if (inst < 0 || inst >= c->n_inst) return DE_EINVAL;
   const GenParams& p = c->bp[inst];
-  cudaError_t e = launch_normalize(p, c->stream);
-  if (e == cudaSuccess && pop_out)
-    e = copy_rows(pop_out, (size_t)p.D * sizeof(float), p.pop0, (size_t)p.pitch * sizeof(float),
-                          (size_t)p.D * sizeof(float), (size_t)p.N, cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess && fit_out)
-    e = cudaMemcpyAsync(fit_out, p.fit, (size_t)p.N * sizeof(float), cudaMemcpyDeviceToHost, c->stream);
-  if (e != cudaSuccess) return DE_ECUDA;
+  if (rows_to_host(p, pop_out, fit_out, c->stream) != cudaSuccess) return DE_ECUDA;
   return sync_stream(c);
 }
 
@@ -523,15 +512,11 @@ int de_batch_set_population(de_ctx* c, int32_t inst, const float* pop, const flo
   if (!c->batch) return DE_ESTATE;
   if (inst < 0 || inst >= c->n_inst) return DE_EINVAL;
   const GenParams& p = c->bp[inst];
-  cudaError_t e = cudaMemsetAsync(p.slots + (size_t)(c->host_gen & 1) * p.N, 0, (size_t)p.N, c->stream);
-  if (e == cudaSuccess)
-    e = copy_rows(p.pop0, (size_t)p.pitch * sizeof(float), pop, (size_t)p.D * sizeof(float),
-                          (size_t)p.D * sizeof(float), (size_t)p.N, cudaMemcpyHostToDevice, c->stream);
+  cudaError_t e = rows_from_host(p, (int)(c->host_gen & 1), pop, fit, c->stream);
   if (e != cudaSuccess) return DE_ECUDA;
   int rc;
   if (fit) {
-    e = cudaMemcpyAsync(p.fit, fit, (size_t)p.N * sizeof(float), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = launch_reset_best(p, c->stream);
+    e = launch_reset_best(p, c->stream);
     if (e == cudaSuccess) e = launch_best_from_fit(p, c->stream);
     if (e == cudaSuccess) e = launch_close_eval(p, c->stream);
     rc = cuda_status(e);

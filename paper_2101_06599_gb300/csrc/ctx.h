@@ -49,8 +49,8 @@ struct de_ctx {
   float* res_pop2 = nullptr;
   std::vector<de_host::Block> blocks;
   std::map<int32_t, cudaGraphExec_t> graphs;
-  void* staging = nullptr;       // device: best row gather
-  void* host_pinned = nullptr;   // host: staging copy and state reads
+  void* staging = nullptr;       // device: best row gather (de_best_async)
+  void* host_pinned = nullptr;   // host, page-locked: best row record and state reads
   size_t host_pinned_bytes = 0;
   long long host_gen = 0;
   // a device error reported by a synchronising call (DE_ETIMEOUT, ...): from
@@ -96,6 +96,23 @@ inline cudaError_t copy_rows(void* dst, size_t dpitch, const void* src, size_t s
   if (dpitch == width && spitch == width) return cudaMemcpyAsync(dst, src, width * rows, kind, s);
   return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, kind, s);
 }
+// Whether a kernel may address all of a host buffer: page-locked and mapped at
+// both ends, on a 16-byte boundary.
+inline bool mapped_host(const void* ptr, size_t bytes) {
+  if (!ptr || ((uintptr_t)ptr & 15u) != 0 || bytes == 0) return false;
+  cudaPointerAttributes a, b;
+  const void* end = static_cast<const char*>(ptr) + bytes - 1;
+  const bool ok = cudaPointerGetAttributes(&a, ptr) == cudaSuccess && a.type == cudaMemoryTypeHost &&
+                  a.devicePointer == ptr && cudaPointerGetAttributes(&b, end) == cudaSuccess &&
+                  b.type == cudaMemoryTypeHost && b.devicePointer == end;
+  cudaGetLastError();
+  return ok;
+}
+// The current rows and their fitness to host memory, and a population (with its
+// fitness, or without) from it into buffer 0, where every row of the generation
+// of this parity then lies.
+cudaError_t rows_to_host(const de::GenParams& p, float* pop, float* fit, cudaStream_t s);
+cudaError_t rows_from_host(const de::GenParams& p, int parity, const float* pop, const float* fit, cudaStream_t s);
 int cuda_status(cudaError_t e);
 void* ctx_alloc(de_ctx* c, size_t bytes);
 void ctx_free(de_ctx* c, void* p);

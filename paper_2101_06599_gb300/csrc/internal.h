@@ -25,11 +25,15 @@ cudaError_t launch_reset_best(const GenParams& p, cudaStream_t s);
 cudaError_t launch_best_from_fit(const GenParams& p, cudaStream_t s);
 // best_f <- value of best_key, best_gen <- gen.
 cudaError_t launch_close_eval(const GenParams& p, cudaStream_t s);
-// staging <- {double f, int64 best_gen, int32 idx, pad, row[D]} of the best row.
+// staging (device or page-locked host) <- {double f, int64 best_gen, int32 idx, pad, row[D]} of the best row.
 cudaError_t launch_best_gather(const GenParams& p, void* staging, cudaStream_t s);
 // Move every row held in slot buffer 1 to slot buffer 0 and clear its slot
 // bit, so that buffer 0 holds the whole population.
 cudaError_t launch_normalize(const GenParams& p, cudaStream_t s);
+// Rows and fitness to and from page-locked host memory (16-byte boundaries; the
+// fitness may be null).
+cudaError_t launch_rows_out(const GenParams& p, float* pop, float* fit, cudaStream_t s);
+cudaError_t launch_rows_in(const GenParams& p, int parity, const float* pop, const float* fit, cudaStream_t s);
 // Test hook: the N x D crossover mask of the generation the context is at.
 cudaError_t launch_debug_mask(const GenParams& p, int xo, uint8_t* mask, cudaStream_t s);
 // Test hook: L of Eq. (9) (table in global and in shared memory) and Alg. 8's
