@@ -22,6 +22,7 @@
 #include "internal.h"
 #include "objectives.cuh"
 #include "ptx.cuh"
+#include "slot_terms.cuh"
 
 namespace de {
 
@@ -161,6 +162,8 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_kernel(const __grid_con
         if (j0 + 2 < p.D) accum_pair(s, t.y, t.z);
         if (j0 + 3 < p.D) accum_pair(s, t.z, t.w);
         if (j0 + 4 < p.D) accum_pair(s, t.w, nb);
+      } else if constexpr (OBJ == kGriewank) {
+        griewank_slot(s, t, j0, p);
       } else {
         accum_gene<OBJ>(s, t.x, j0, p);
         if (j0 + 1 < p.D) accum_gene<OBJ>(s, t.y, j0 + 1, p);

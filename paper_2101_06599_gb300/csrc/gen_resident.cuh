@@ -51,6 +51,7 @@
 #include "internal.h"
 #include "objectives.cuh"
 #include "ptx.cuh"
+#include "slot_terms.cuh"
 
 namespace de {
 
@@ -126,7 +127,7 @@ __host__ __device__ inline ResLayout res_layout(bool seg, int rpc, int D4, int g
 }
 
 // One slot q of a row (genes 4q ..) added to a thread's sums; nb is gene 4q + 4.
-template <int OBJ>
+template <bool kSeg, int OBJ>
 __device__ __forceinline__ void res_slot(Acc& a, const float4& x, float nb, int q, const GenParams& p) {
   const int j0 = 4 * q;
   if constexpr (OBJ == kRosenbrock) {
@@ -134,6 +135,8 @@ __device__ __forceinline__ void res_slot(Acc& a, const float4& x, float nb, int 
     if (j0 + 2 < p.D) accum_pair(a, x.y, x.z);
     if (j0 + 3 < p.D) accum_pair(a, x.z, x.w);
     if (j0 + 4 < p.D) accum_pair(a, x.w, nb);
+  } else if constexpr (kSeg && OBJ == kGriewank) {
+    griewank_slot(a, x, j0, p);
   } else {
     accum_gene<OBJ>(a, x.x, j0, p);
     if (j0 + 1 < p.D) accum_gene<OBJ>(a, x.y, j0 + 1, p);
@@ -362,7 +365,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         if constexpr (OBJ == kRosenbrock) {
           if (q + 1 < p.D4) nb = ((q + 1 >= a0 && q + 1 <= b0) || q + 1 <= b1) ? tr[q + 1].x : x[q + 1].x;
         }
-        res_slot<OBJ>(s, xv, nb, q, p);
+        res_slot<kSeg, OBJ>(s, xv, nb, q, p);
       }
       to[32 * w + lane] = s.a;
       if (NS > 1) to[T + 32 * w + lane] = s.b;
@@ -445,7 +448,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
           // against 2.4 at N = 50, D = 10, and a __syncwarp alone does not help
           if constexpr (OBJ != kRosenbrock) (void)__shfl_down_sync(0xFFFFFFFFu, te.x, 1);
           __syncwarp();
-          res_slot<OBJ>(es, te, nx, qe, p);
+          res_slot<kSeg, OBJ>(es, te, nx, qe, p);
           __syncwarp();
 #pragma unroll 1
           for (uint32_t todo = pl.again; todo; todo &= todo - 1u) {
@@ -602,7 +605,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
             if (lane == 31) nb = (pw + 1 < nw) ? first[v * 8 + pw + 1] : (v + 1 < V ? first[(v + 1) * 8] : 0.0f);
           }
           const int q = pw * 32 + lane + v * T;
-          if (q < p.D4) res_slot<OBJ>(s, x[v], nb, q, p);
+          if (q < p.D4) res_slot<kSeg, OBJ>(s, x[v], nb, q, p);
         }
         res_butterfly<NS, 16>(s);
         if (W > 1) {
