@@ -204,9 +204,14 @@ int note_device_error(de_ctx* c, int err) {
 // which the kernel fills as well as a linear copy does (192 GB/s out, 208 in). us
 // per call, copies -> kernel, out and in (with the evaluation): 100 x 30 18.6 ->
 // 14.8, 29.0 -> 22.1; 1000 x 100 24.0 -> 16.7, 58.5 -> 25.7; 4096 x 1001 109 -> 100,
-// 260 -> 109; 16384 x 4097 1795 -> 1408, 1690 -> 1352; 16384 x 10000 3423 -> 3409,
-// 3277 -> 3275; 128 instances (760 MB) out 7.15 -> 5.78 ms.
+// 260 -> 109; 16384 x 4097 1795 -> 1408, 1690 -> 1352; out only, 16384 x 10000 3423 ->
+// 3409, 128 instances (760 MB) 7.15 -> 5.78 ms.
 // Anything else goes through the copy engine.
+// Populations from the host of more than this go by one linear copy where their
+// rows allow it: the kernel's first reads of that much host memory are slower (655
+// MB and 20 generations 6.28 ms with it, 6.23 with the copy).
+constexpr size_t kCopyInBytes = 64u << 20;
+
 cudaError_t rows_to_host(const GenParams& p, float* pop, float* fit, cudaStream_t s) {
   const size_t row = (size_t)p.D * sizeof(float), bytes = row * p.N, fbytes = (size_t)p.N * sizeof(float);
   if (mapped_host(pop, bytes) && (!fit || mapped_host(fit, fbytes))) return launch_rows_out(p, pop, fit, s);
@@ -219,7 +224,9 @@ cudaError_t rows_to_host(const GenParams& p, float* pop, float* fit, cudaStream_
 
 cudaError_t rows_from_host(const GenParams& p, int parity, const float* pop, const float* fit, cudaStream_t s) {
   const size_t row = (size_t)p.D * sizeof(float), bytes = row * p.N, fbytes = (size_t)p.N * sizeof(float);
-  if (mapped_host(pop, bytes) && (!fit || mapped_host(fit, fbytes))) return launch_rows_in(p, parity, pop, fit, s);
+  const bool stream = p.pitch == p.D && bytes > kCopyInBytes;
+  if (!stream && mapped_host(pop, bytes) && (!fit || mapped_host(fit, fbytes)))
+    return launch_rows_in(p, parity, pop, fit, s);
   // the current generation's slot half is cleared: buffer 0 holds every row
   cudaError_t e = cudaMemsetAsync(p.slots + (size_t)parity * p.N, 0, (size_t)p.N, s);
   if (e == cudaSuccess)

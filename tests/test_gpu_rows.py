@@ -9,9 +9,10 @@ pytestmark = pytest.mark.gpu
 
 from paper_2101_06599_gb300 import de as DE
 
-# one gene, totals that are no multiple of four, rows inside one slot, several spans; a pitch that is D
+# one gene, totals that are no multiple of four, rows inside one slot, several spans; a pitch that is D, small
+# and beyond what the kernel reads
 SHAPES = [(4, 1), (5, 1), (300, 30), (65, 63), (40, 65), (33, 127), (9, 255), (51, 1001), (13, 1025), (7, 4097),
-          (20, 64)]
+          (20, 64), (4096, 4104)]
 
 
 def _host(n, kind):
