@@ -189,7 +189,7 @@ int de_step(de_ctx *ctx);
  * de_step bit for bit; the first such run takes two more population buffers
  * from the allocator (without them, and on a capturing stream, every
  * generation is a launch). The waits between rows in that launch give up
- * after 1 s (DE_ETIMEOUT). */
+ * after 1 s or the limit that de_set_wait_limit gives (DE_ETIMEOUT). */
 int de_run(de_ctx *ctx, int32_t generations);
 
 /* Capture and instantiate the graph that de_run(ctx, generations) replays,
@@ -207,7 +207,8 @@ int de_synchronize(de_ctx *ctx);
 
 /* Limit, in nanoseconds of the GPU's global timer, of the device waits that
  * guard no copy or tensor-core operation in flight: the grid barrier of the
- * batched one-launch generation between its row plans and its rows. ns = 0
+ * batched one-launch generation between its row plans and its rows, and the
+ * waits between rows in the launches of de_run that make many generations. ns = 0
  * restores the default (1 s); DE_EINVAL for ns < 0. A CTA whose barrier wait
  * gives up records DE_ETIMEOUT and takes no rows; the CTAs the barrier
  * released process every row between them, so the generation is still

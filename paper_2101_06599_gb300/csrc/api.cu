@@ -491,6 +491,7 @@ static cudaGraphExec_t run_graph(de_ctx* c, int32_t generations) {
     rp.words = c->res_words;
     rp.pop2 = c->res_pop2;
     rp.row_threads = c->block;
+    rp.wait_ns = c->wait_ns ? c->wait_ns : kWaitLimitNs;
     for (int32_t left = generations; left > 0 && le == cudaSuccess; left -= rp.gens) {
       rp.gens = std::min(left, kResMaxGens);
       le = shape.cluster ? launch_cluster(c->xo, c->obj, c->p, rp.gens, &c->res_state->hist, c->stream)

@@ -56,7 +56,7 @@ struct de_ctx {
   // a device error reported by a synchronising call (DE_ETIMEOUT, ...): from
   // then on calls that would launch generations return DE_ESTATE
   int failed = 0;
-  unsigned long long wait_ns = 0;   // batched grid-barrier limit (0: the 1 s default)
+  unsigned long long wait_ns = 0;   // limit of the waits that guard nothing in flight (0: the 1 s default)
   // batched contexts (de_batch_create); the fields above then describe nothing
   bool batch = false;
   int n_inst = 0;

@@ -36,8 +36,11 @@
 //    O(D). Binomial rows take a warp per 128 genes and sum all. Both sum in
 //    gen_kernel's order, so values, selections and populations are
 //    bit-identical to de_step's.
-//  - Every wait is bounded (kWaitLimitNs); a CTA that gives up records
-//    DE_ETIMEOUT, leaves the loop and still closes, so the launch ends.
+//  - Every wait is bounded (ResidentParams::wait_ns); a CTA that gives up
+//    records DE_ETIMEOUT, leaves the loop and still closes, so the launch ends.
+//    Whether a wait was met is one answer for a warp, and for the warps of a row
+//    one that they agree on at the row's barriers: no plan, word or barrier is
+//    used by lanes or warps that went on alone.
 //
 // What bounds it: latency. A generation is the chain poll a word (L2, 0.5 us on
 // a line that another SM has just written), load the genes (0.5 us), some 300
@@ -163,7 +166,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
   const GenParams& p = rp.g;
   extern __shared__ __align__(16) unsigned char res_smem[];
   __shared__ int s_dead, s_drawn, s_safe;   // a wait gave up; generations drawn; last generation whose trials may be stored
-  __shared__ int s_done[kResWarps], s_stop[kResWarps];   // per group: generations finished; it ends early
+  __shared__ int s_done[kResWarps];         // per group: generations finished
   __shared__ unsigned long long s_masked, s_wins, s_key, s_hist;
 
   constexpr int NS = ObjTraits<OBJ>::kSums;
@@ -208,10 +211,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     s_key = ~0ULL;
     s_hist = ~0ULL;
   }
-  if (tid < kResWarps) {
-    s_done[tid] = 0;
-    s_stop[tid] = 0;
-  }
+  if (tid < kResWarps) s_done[tid] = 0;
   __syncthreads();
 
   const int depth = res_depth(rp.rpc);             // a power of two
@@ -251,9 +251,15 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
       plans[(size_t)(k & (depth - 1)) * rp.rpc + l] = pl;
     }
   };
+  // called by a whole warp, with one answer for it
+  auto dead = [&] { return __shfl_sync(0xFFFFFFFFu, ld_flag(&s_dead), 0) != 0; };
+  auto late = [&](unsigned long long t0) { return __any_sync(0xFFFFFFFFu, global_ns() - t0 > rp.wait_ns) != 0; };
   auto give_up = [&] {
-    st_flag(&s_dead, 1);
-    atomicMax(&p.st->error, 4u);                   // DE_ETIMEOUT
+    if (lane == 0) {
+      st_flag(&s_dead, 1);
+      atomicMax(&p.st->error, 4u);                 // DE_ETIMEOUT
+    }
+    __syncwarp();
   };
   auto finished = [&] {                            // generations that every group of this CTA has finished
     return (int)__reduce_min_sync(0xFFFFFFFFu, lane < groups ? (unsigned)ld_flag(&s_done[lane]) : 0x7FFFFFFFu);
@@ -261,7 +267,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
   if (helper == 1) {                               // draws ahead
     const int batch = max(1, min(32 / max(1, rows), depth / 2));
     unsigned long long t0 = global_ns();
-    for (int k = 0; k < rp.gens && !ld_flag(&s_dead);) {
+    for (int k = 0; k < rp.gens && !dead();) {
       const int room = min(depth - (k - finished()), rp.gens - k);
       if (room >= min(batch, rp.gens - k)) {
         draw(k, min(room, batch));
@@ -269,7 +275,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         __syncwarp();
         if (lane == 0) st_flag(&s_drawn, k);
         t0 = global_ns();
-      } else if (__any_sync(0xFFFFFFFFu, global_ns() - t0 > kWaitLimitNs)) {
+      } else if (late(t0)) {
         give_up();
       } else {
         __nanosleep(200);                          // leaves the issue slots to the rows
@@ -278,7 +284,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
   } else if (helper == 2) {                        // counts finished generations: this CTA's, and everyone's
     int arrived = 0, all = 0;
     unsigned long long t0 = global_ns();
-    while (all < rp.gens && !ld_flag(&s_dead)) {
+    while (all < rp.gens && !dead()) {
       bool moved = false;
       for (const int done = finished(); arrived < done; ++arrived, moved = true)
         if (lane == 0) red_release(&rp.rs->ctr[arrived & 7], 1u);
@@ -288,47 +294,55 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         if (lane == 0) st_flag(&s_safe, all + 2);
         moved = true;
       }
-      const unsigned long long now = global_ns();
-      if (moved) t0 = now;
-      else if (__any_sync(0xFFFFFFFFu, now - t0 > kWaitLimitNs)) give_up();
+      if (moved) t0 = global_ns();
+      else if (late(t0)) give_up();
       else __nanosleep(64);
     }
   }
-  // a worker's wait until `flag` (in shared memory) is at least `want`; `seen`
-  // is the last value read, so that most waits read nothing
+  // a worker warp's wait until `flag` (in shared memory) is at least `want`;
+  // `seen` is the last value read, so that most waits read nothing. False: the
+  // wait, or another one of the CTA, gave up, and what the flag stands for is not there
   int drawn_seen = 0, safe_seen = 2;
   auto wait_flag = [&](const int* flag, int& seen, int want) {
-    if (seen >= want) return;
+    if (seen >= want) return true;
     const unsigned long long t0 = global_ns();
     for (int n = 0;; ++n) {
       seen = __shfl_sync(0xFFFFFFFFu, ld_flag(flag), 0);
-      if (seen >= want || ld_flag(&s_dead)) break;
-      if ((n & 1023) == 1023 && global_ns() - t0 > kWaitLimitNs) give_up();
+      if (seen >= want) break;
+      if (dead()) return false;
+      if ((n & 1023) == 1023 && late(t0)) give_up();
     }
     __threadfence_block();
     __syncwarp();
+    return true;
   };
 
   // the buffers that hold the rows of a generation's donors: lanes 0-2 wait for
-  // the words of row pl.r[lane] and the result is every lane's
+  // the words of row pl.r[lane] and the result is every lane's. False: gave up
   auto donors = [&](const ResPlan& pl, uint32_t tag, const float4*& d1, const float4*& d2, const float4*& d3) {
-    uint32_t buf = 0u;
+    uint32_t w = 0u, ahead = 0u;
+    const uint32_t* wp = rp.words + (size_t)(lane == 0 ? pl.r[0] : (lane == 1 ? pl.r[1] : pl.r[2])) * kResWordStride;
     if (lane < 3) {
-      const uint32_t* wp = rp.words + (size_t)(lane == 0 ? pl.r[0] : (lane == 1 ? pl.r[1] : pl.r[2])) * kResWordStride;
-      uint32_t w = ld_acquire(wp), ahead = ((w >> 8) - tag) & kResTagMask;
-      if (ahead > 3u) {
-        const unsigned long long t0 = global_ns();
-        for (int n = 0; ahead > 3u && !ld_flag(&s_dead); ++n) {
+      w = ld_acquire(wp);
+      ahead = ((w >> 8) - tag) & kResTagMask;
+    }
+    if (__any_sync(0xFFFFFFFFu, ahead > 3u)) {
+      const unsigned long long t0 = global_ns();
+      for (int n = 0;; ++n) {
+        if (ahead > 3u) {
           w = ld_acquire(wp);
           ahead = ((w >> 8) - tag) & kResTagMask;
-          if ((n & 63) == 63 && global_ns() - t0 > kWaitLimitNs) give_up();
         }
+        if (!__any_sync(0xFFFFFFFFu, ahead > 3u)) break;
+        if (dead()) return false;
+        if ((n & 63) == 63 && late(t0)) give_up();
       }
-      buf = (w >> (2u * min(ahead, 3u))) & 3u;
     }
+    const uint32_t buf = (w >> (2u * ahead)) & 3u;
     d1 = reinterpret_cast<const float4*>(buffer(__shfl_sync(0xFFFFFFFFu, buf, 0)) + (size_t)pl.r[0] * p.pitch);
     d2 = reinterpret_cast<const float4*>(buffer(__shfl_sync(0xFFFFFFFFu, buf, 1)) + (size_t)pl.r[1] * p.pitch);
     d3 = reinterpret_cast<const float4*>(buffer(__shfl_sync(0xFFFFFFFFu, buf, 2)) + (size_t)pl.r[2] * p.pitch);
+    return true;
   };
 
   unsigned long long masked = 0, wins = 0, key = ~0ULL, hist = ~0ULL;
@@ -387,8 +401,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     }
     for (int k = 0; k < rp.gens && helper < 1; ++k) {
       const uint32_t tag = (tag0 + (uint32_t)k) & kResTagMask;
-      wait_flag(&s_drawn, drawn_seen, k + 1);
-      for (int l = grp; l < rows; l += groups) {
+      bool ok = wait_flag(&s_drawn, drawn_seen, k + 1);
+      for (int l = grp; l < rows && ok; l += groups) {
         const ResPlan pl = plans[(size_t)(k & (depth - 1)) * rp.rpc + l];
         const float fi = sfit[l];
         const uint32_t sl = sslot[l];
@@ -407,7 +421,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         // version of the row and the segment leaves as it is
         uint32_t stale = sstale[l * 32 + lane];
         const uint32_t nshift = 8u * ((sl >> 2) & 3u), old = (stale >> nshift) & 0xFFu;
-        wait_flag(&s_safe, safe_seen, k);
+        ok = wait_flag(&s_safe, safe_seen, k);
+        if (!ok) break;
 #pragma unroll 1
         for (uint32_t todo = __reduce_or_sync(0xFFFFFFFFu, old); todo; todo &= todo - 1u) {
           const int w = __ffs((int)todo) - 1, q = 32 * w + lane;
@@ -428,7 +443,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         float4 te = x[qe];
         Acc es{0.0f, 0.0f, 0.0f};
         const float4 *d1, *d2, *d3;
-        donors(pl, tag, d1, d2, d3);
+        ok = donors(pl, tag, d1, d2, d3);
+        if (!ok) break;
         if (brief) {
           if (mine) {
             const float4 a1 = ld_l2(d1 + qe), a2 = ld_l2(d2 + qe), a3 = ld_l2(d3 + qe);
@@ -531,18 +547,20 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         }
         __syncwarp();
       }
+      if (!ok) break;
       if (lane == 0) st_flag(&s_done[grp], k + 1);
-      if (__any_sync(0xFFFFFFFFu, ld_flag(&s_dead))) break;
     }
   } else {
     float* red = reinterpret_cast<float*>(res_smem + lay.red) + grp * 2 * 24;
     float* first = reinterpret_cast<float*>(res_smem + lay.first) + grp * V * 8;
     int set = 0;
+    // whether every warp of the group has what it waited for; a barrier of them
+    auto agree = [&](bool ok) { return W > 1 ? named_bar_and(1 + grp, 32 * W, ok) : ok; };
     for (int k = 0; k < rp.gens && helper < 1; ++k) {
       const uint32_t g = (uint32_t)(gen0 + k), tag = (tag0 + (uint32_t)k) & kResTagMask;
-      wait_flag(&s_drawn, drawn_seen, k + 1);
+      bool ok = wait_flag(&s_drawn, drawn_seen, k + 1);   // a warp without its plan goes on to the barrier
       for (int l = grp; l < rows; l += groups) {
-        const ResPlan pl = plans[(size_t)(k & (depth - 1)) * rp.rpc + l];
+        const ResPlan pl = ok ? plans[(size_t)(k & (depth - 1)) * rp.rpc + l] : ResPlan{};
         const int i = row0 + l;
         const float fi = sfit[l];
         const uint32_t sl = sslot[l];
@@ -553,16 +571,16 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         for (int s = 0; s < V; ++s) {
           const int q = pw * 32 + lane + s * T;
           x[s] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-          if (q < p.D4) {
+          if (ok && q < p.D4) {
             unsigned b = bin_mask(p, philox_block_rk(p.rk, kStreamBin, p.inst, g, (uint32_t)i, (uint32_t)q), q, pl.jrand);
             b &= (1u << min(4, p.D - 4 * q)) - 1u;
             m |= b << (4 * s);
             x[s] = sx[l * p.D4 + q];
           }
         }
-        masked += (unsigned)__popc(m);
         const float4 *d1 = nullptr, *d2 = nullptr, *d3 = nullptr;
-        if (__any_sync(0xFFFFFFFFu, m != 0u)) donors(pl, tag, d1, d2, d3);
+        if (__any_sync(0xFFFFFFFFu, m != 0u)) ok = donors(pl, tag, d1, d2, d3);
+        if (!ok) m = 0u;
         uint32_t touched = 0u;
 #pragma unroll
         for (int s = 0; s < V; ++s) {
@@ -581,11 +599,13 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         // buffer holds from an older version
         uint32_t stale = sstale[(l * W + pw) * 32 + lane];
         const uint32_t nshift = 8u * ((sl >> 2) & 3u), put = ((stale >> nshift) & 0xFFu) | touched;
-        wait_flag(&s_safe, safe_seen, k);
+        ok = ok && wait_flag(&s_safe, safe_seen, k);
+        if (ok) {
 #pragma unroll
-        for (int s = 0; s < V; ++s) {
-          const int q = pw * 32 + lane + s * T;
-          if (((put >> s) & 1u) && q < p.D4) __stcg(out + q, x[s]);
+          for (int s = 0; s < V; ++s) {
+            const int q = pw * 32 + lane + s * T;
+            if (((put >> s) & 1u) && q < p.D4) __stcg(out + q, x[s]);
+          }
         }
         // fitness, in block_row_fitness's order
         if constexpr (OBJ == kRosenbrock) {
@@ -615,7 +635,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
             if (NS > 1) r[8 + pw] = s.b;
             if (NS > 2) r[16 + pw] = s.c;
           }
-          named_bar_sync(1 + grp, 32 * W);         // and every store of the trial precedes the row's word
+          ok = agree(ok);                          // and every store of the trial precedes the row's word
           set ^= 1;                                // this set's readers are past the next barrier before it is reused
           const bool in = (lane & 7) < nw;
           s.a = in ? r[lane & 7] : 0.0f;
@@ -629,7 +649,9 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         }
         float f = finalize_fitness<OBJ>(s, p);
         if (f != f) f = __int_as_float(0x7F800000);
+        if (!ok) break;
         const bool win = f < fi;
+        masked += (unsigned)__popc(m);
         if (pw == 0 && lane == 0) decide(k, tag, l, sl, f, win);
         // a winner's buffer holds the row, the others miss its slots; a loser's
         // buffer misses the slots that it tried
@@ -646,11 +668,9 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
       }
       // the group's reads of generation k are over once its warps are here; they
       // end early together or not at all
-      if (pw == 0 && lane == 0) s_stop[grp] = ld_flag(&s_dead);
-      if (W > 1) named_bar_sync(1 + grp, 32 * W);
-      else __syncwarp();
+      __syncwarp();
+      if (!agree(ok)) break;
       if (pw == 0 && lane == 0) st_flag(&s_done[grp], k + 1);
-      if (s_stop[grp]) break;
     }
   }
 

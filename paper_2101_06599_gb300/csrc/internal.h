@@ -70,6 +70,7 @@ struct ResidentParams {
   int rpc;                     // rows per CTA
   int row_threads;             // threads per row in gen_kernel's order
   int groups, xo;              // rows a CTA processes at a time; crossover
+  unsigned long long wait_ns;  // limit of each wait
 };
 struct ResidentShape {
   int grid, block, rpc, groups;
