@@ -212,7 +212,11 @@ int de_synchronize(de_ctx *ctx);
  * restores the default (1 s); DE_EINVAL for ns < 0. A CTA whose barrier wait
  * gives up records DE_ETIMEOUT and takes no rows; the CTAs the barrier
  * released process every row between them, so the generation is still
- * complete and identical to one without the timeout. The waits of the
+ * complete and identical to one without the timeout. A launch of many
+ * generations that gives up ends with whole rows and their fitness: g
+ * generations are counted, and every row is that of generation g, g + 1, g + 2
+ * or g + 3 of a run without the timeout; launches of such a run that were queued
+ * behind it do nothing. The waits of the
  * pipelined and tensor-core kernels, which guard bulk copies and MMAs in
  * flight, keep their fixed 1 s limit. de_get_wait_limit reports the limit
  * in force. Drops the context's captured graphs. */

@@ -38,6 +38,9 @@
 //    bit-identical to de_step's.
 //  - Every wait is bounded (ResidentParams::wait_ns); a CTA that gives up
 //    records DE_ETIMEOUT, leaves the loop and still closes, so the launch ends.
+//    Its rows stay where their words say; the last CTA, when nobody reads any
+//    more, brings every row's last version together and counts the generations
+//    that all rows have finished.
 //    Whether a wait was met is one answer for a warp, and for the warps of a row
 //    one that they agree on at the row's barriers: no plan, word or barrier is
 //    used by lanes or warps that went on alone.
@@ -168,6 +171,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
   __shared__ int s_dead, s_drawn, s_safe;   // a wait gave up; generations drawn; last generation whose trials may be stored
   __shared__ int s_done[kResWarps];         // per group: generations finished
   __shared__ unsigned long long s_masked, s_wins, s_key, s_hist;
+  __shared__ int s_last, s_least;           // this CTA closes; generations that every row has finished
 
   constexpr int NS = ObjTraits<OBJ>::kSums;
   const int T = rp.row_threads, nw = T >> 5;       // threads and warps of a row in gen_kernel's order
@@ -186,7 +190,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
   const int row0 = blockIdx.x * rp.rpc;
   const int rows = min(rp.rpc, p.N - row0);
   const long long gen0 = p.st->gen;
-  const uint32_t tag0 = rp.rs->epoch;
+  const uint32_t tag0 = rp.rs->epoch, gave_up = rp.rs->failed;
   auto buffer = [&](uint32_t b) { return b == 0 ? p.pop0 : (b == 1 ? p.pop1 : rp.pop2 + (size_t)(b - 2) * p.N * p.pitch); };
 
   const uint8_t* slot_in = p.slots + (size_t)(gen0 & 1) * p.N;
@@ -194,6 +198,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     const int l = q / p.D4, i = row0 + l;
     sx[q] = reinterpret_cast<const float4*>((slot_in[i] ? p.pop1 : p.pop0) + (size_t)i * p.pitch)[q - l * p.D4];
   }
+  if (gave_up) return;                             // a launch before this one did
   for (int q = tid; q < rows * W * 32; q += blockDim.x)
     sstale[q] = slot_in[row0 + q / (W * 32)] ? 0xFFFF00FFu : 0xFFFFFF00u;
   for (int l = tid; l < rows; l += blockDim.x) {
@@ -210,6 +215,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     s_wins = 0ULL;
     s_key = ~0ULL;
     s_hist = ~0ULL;
+    s_least = rp.gens;
   }
   if (tid < kResWarps) s_done[tid] = 0;
   __syncthreads();
@@ -674,8 +680,9 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     }
   }
 
-  // the run's state, once nobody reads the buffers any more: rows to buffer 0,
-  // fitness, slot bytes, counters; the last CTA closes
+  // the run's state: rows to buffer 0, fitness, slot bytes, counters; the last
+  // CTA closes. Unless this CTA gave up, its second helper has seen every CTA
+  // finish every generation, and nobody reads the buffers any more
   if (masked) atomicAdd(&s_masked, masked);
   if (wins) atomicAdd(&s_wins, wins);
   if (key != ~0ULL) {
@@ -683,15 +690,18 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     atomicMin(&s_hist, hist);
   }
   __syncthreads();
-  for (int q = tid; q < rows * p.D4; q += blockDim.x) {
-    const int l = q / p.D4;
-    reinterpret_cast<float4*>(p.pop0 + (size_t)(row0 + l) * p.pitch)[q - l * p.D4] = sx[q];
+  if (!s_dead) {
+    for (int q = tid; q < rows * p.D4; q += blockDim.x) {
+      const int l = q / p.D4;
+      reinterpret_cast<float4*>(p.pop0 + (size_t)(row0 + l) * p.pitch)[q - l * p.D4] = sx[q];
+    }
   }
   uint8_t* slot_out = p.slots + (size_t)((gen0 + rp.gens) & 1) * p.N;
   for (int l = tid; l < rows; l += blockDim.x) {
     p.fit[row0 + l] = sfit[l];
     slot_out[row0 + l] = 0;
   }
+  __syncthreads();
   if (tid == 0) {
     atomicAdd(&p.st->masked, s_masked);
     if (s_wins) {
@@ -700,20 +710,37 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
       atomicMin(&rp.rs->hist, s_hist);
     }
     __threadfence();
-    if (atomicAdd(&p.st->done, 1u) == gridDim.x - 1) {
-      __threadfence();
-      const unsigned long long bk = atomicAdd(&p.st->best_key, 0ULL), h = atomicExch(&rp.rs->hist, ~0ULL);
-      const float bf = from_ordered_bits((uint32_t)(bk >> 32));
-      if (bf < p.st->best_f) {
-        p.st->best_f = bf;
-        p.st->best_gen = gen0 + (long long)(uint32_t)h;   // the first generation that reached the best value
-      }
-      p.st->gen = gen0 + rp.gens;
-      p.st->base_row = (int)(uint32_t)(bk & 0xFFFFFFFFull);
-      p.st->done = 0u;
-      rp.rs->epoch = (tag0 + (uint32_t)rp.gens + 1u) & kResTagMask;
-      for (int c = 0; c < 8; ++c) rp.rs->ctr[c] = 0u;
+    s_last = atomicAdd(&p.st->done, 1u) == gridDim.x - 1 ? 1 : 0;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_last) return;
+  const bool failed = ld_acquire(&p.st->error) != 0u;
+  if (failed) {
+    for (int i = tid >> 5; i < p.N; i += (int)blockDim.x >> 5) {   // a warp per row
+      const uint32_t w = ld_acquire(rp.words + (size_t)i * kResWordStride);
+      const float4* from = reinterpret_cast<const float4*>(buffer(w & 3u) + (size_t)i * p.pitch);
+      float4* to = reinterpret_cast<float4*>(p.pop0 + (size_t)i * p.pitch);
+      if (w & 3u)
+        for (int q = lane; q < p.D4; q += 32) to[q] = ld_l2(from + q);
+      if (lane == 0) atomicMin(&s_least, (int)(((w >> 8) - tag0) & kResTagMask));
     }
+    for (int i = tid; i < 2 * p.N; i += blockDim.x) p.slots[i] = 0;
+    __syncthreads();
+  }
+  if (tid == 0) {
+    const unsigned long long bk = atomicAdd(&p.st->best_key, 0ULL), h = atomicExch(&rp.rs->hist, ~0ULL);
+    const float bf = from_ordered_bits((uint32_t)(bk >> 32));
+    if (bf < p.st->best_f) {
+      p.st->best_f = bf;
+      p.st->best_gen = gen0 + min((long long)(uint32_t)h, (long long)s_least);   // the first generation that reached the best value
+    }
+    p.st->gen = gen0 + s_least;
+    p.st->base_row = (int)(uint32_t)(bk & 0xFFFFFFFFull);
+    p.st->done = 0u;
+    rp.rs->epoch = (tag0 + (uint32_t)rp.gens + 1u) & kResTagMask;
+    rp.rs->failed = failed ? 1u : 0u;
+    for (int c = 0; c < 8; ++c) rp.rs->ctr[c] = 0u;
   }
 }
 

@@ -55,7 +55,7 @@ constexpr int kResWordStride = 32;   // a row word has a 128-byte line of its ow
 constexpr int kResMaxGens = 4096;
 struct ResState {
   unsigned epoch;              // row tag that the next launch starts at (tags do not repeat between launches)
-  unsigned pad_;
+  unsigned failed;             // a launch gave up: the ones queued behind it do nothing
   unsigned long long hist;     // (orderable best value of the run << 32) | first generation that reached it
   unsigned pad2_[28];
   unsigned ctr[8];             // CTAs that finished generation k, k mod 8, on a line of their own; zero between launches

@@ -44,3 +44,35 @@ def test_a_wait_that_gives_up_ends_the_run(N, D, xo, obj):
         assert u.tobytes() == v.tobytes()
     b.close()
     c.close()
+
+
+def _generation_and_error(a):
+    """Generations counted and the device error, from a checkpoint (the other calls report the error alone)."""
+    blob = np.frombuffer(a.save(), np.uint8)
+    st = blob[72:]                               # magic .. repair; then best_key, gen, best_gen, 3 counters, done, error
+    return int(st[8:16].view(np.int64)[0]), int(st[16:24].view(np.int64)[0]), int(st[52:56].view(np.uint32)[0])
+
+
+@pytest.mark.parametrize("limit", [1, 3000, 30000])
+@pytest.mark.parametrize("N,D,xo,obj", CASES)
+def test_what_a_run_that_gave_up_leaves(N, D, xo, obj, limit):
+    """Whole rows with their fitness, each of the counted generation or one of the
+    three after it (bit for bit), and nothing from what was queued behind it."""
+    a, b = _optimizer(N, D, xo, obj), _optimizer(N, D, xo, obj)
+    b.set_kernel(1)
+    DE.de_set_wait_limit(a.ctx, limit)
+    a.run(300)
+    a.run(300)                                   # behind a launch that gave up: does nothing
+    x, f = a.population()
+    g, best_gen, err = _generation_and_error(a)
+    assert err == (0 if g == 600 else DE.DE_ETIMEOUT) and best_gen <= g
+    assert err or limit > 1
+    b.run(g)
+    there = np.zeros(N, bool)
+    for k in range(4 if err else 1):
+        y, fy = b.population()
+        there |= np.all(x.view(np.uint32) == y.view(np.uint32), axis=1) & (f.view(np.uint32) == fy.view(np.uint32))
+        b.step()
+    assert there.all()
+    a.close()
+    b.close()
