@@ -97,7 +97,7 @@ __device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
 }
 __device__ __forceinline__ int ld_flag(const int* p) {   // flags in shared memory
   int v;
-  asm volatile("ld.relaxed.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_flag(int* p, int v) {
@@ -267,8 +267,13 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     }
     __syncwarp();
   };
-  auto finished = [&] {                            // generations that every group of this CTA has finished
-    return (int)__reduce_min_sync(0xFFFFFFFFu, lane < groups ? (unsigned)ld_flag(&s_done[lane]) : 0x7FFFFFFFu);
+  // generations that every group of this CTA has finished. Each lane acquires its
+  // group's flag and the warp's barrier hands that on: what the warp then writes,
+  // or lane 0 releases, comes after the groups' reads
+  auto finished = [&] {
+    const int n = (int)__reduce_min_sync(0xFFFFFFFFu, lane < groups ? (unsigned)ld_flag(&s_done[lane]) : 0x7FFFFFFFu);
+    __syncwarp();
+    return n;
   };
   if (helper == 1) {                               // draws ahead
     const int batch = max(1, min(32 / max(1, rows), depth / 2));
@@ -296,6 +301,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         if (lane == 0) red_release(&rp.rs->ctr[arrived & 7], 1u);
       const uint32_t have = ld_acquire(&rp.rs->ctr[all & 7]);
       if (__all_sync(0xFFFFFFFFu, have >= (uint32_t)((all >> 3) + 1) * gridDim.x)) {
+        __syncwarp();
         ++all;
         if (lane == 0) st_flag(&s_safe, all + 2);
         moved = true;
@@ -318,7 +324,6 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
       if (dead()) return false;
       if ((n & 1023) == 1023 && late(t0)) give_up();
     }
-    __threadfence_block();
     __syncwarp();
     return true;
   };
@@ -344,6 +349,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         if ((n & 63) == 63 && late(t0)) give_up();
       }
     }
+    __syncwarp();                                  // what lanes 0-2 acquired, the others may read
     const uint32_t buf = (w >> (2u * ahead)) & 3u;
     d1 = reinterpret_cast<const float4*>(buffer(__shfl_sync(0xFFFFFFFFu, buf, 0)) + (size_t)pl.r[0] * p.pitch);
     d2 = reinterpret_cast<const float4*>(buffer(__shfl_sync(0xFFFFFFFFu, buf, 1)) + (size_t)pl.r[1] * p.pitch);
