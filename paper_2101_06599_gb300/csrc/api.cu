@@ -12,6 +12,8 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
 #include "ctx.h"
 
 using namespace de_host;
@@ -197,6 +199,39 @@ int note_device_error(de_ctx* c, int err) {
   return err;
 }
 
+// A buffer may span several page-locked allocations or registrations, with
+// memory between them that is neither: each one's range is looked up, the next
+// where it ends, until they cover the buffer (in pieces of 64 at most; a program's
+// buffer is one).
+bool mapped_host(const void* ptr, size_t bytes) {
+  if (!ptr || ((uintptr_t)ptr & 15u) != 0 || bytes == 0) return false;
+  using GetAttribute = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+  static const GetAttribute get = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    const bool ok = cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q) ==
+                        cudaSuccess && q == cudaDriverEntryPointSuccess;
+    cudaGetLastError();
+    return reinterpret_cast<GetAttribute>(ok ? f : nullptr);
+  }();
+  if (!get) return false;
+  uintptr_t at = (uintptr_t)ptr;
+  const uintptr_t end = at + bytes;
+  for (int k = 0; k < 64 && at < end; ++k) {
+    cudaPointerAttributes a;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    const bool ok = cudaPointerGetAttributes(&a, (const void*)at) == cudaSuccess && a.type == cudaMemoryTypeHost &&
+                    a.devicePointer == (const void*)at &&
+                    get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)at) == CUDA_SUCCESS &&
+                    get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, (CUdeviceptr)at) == CUDA_SUCCESS;
+    if (!ok || start > at || start + size <= at) break;
+    at = start + size;
+  }
+  cudaGetLastError();
+  return at >= end;
+}
+
 // Page-locked buffers are written and read by a kernel: one launch in place of
 // the move of the rows of buffer 1, two copies (rows of D % 8 != 0 in 2D) and,
 // for a population from the host, the clearing of the slot bytes. Small calls are
@@ -219,6 +254,7 @@ cudaError_t rows_to_host(const GenParams& p, float* pop, float* fit, cudaStream_
   if (e == cudaSuccess && pop)
     e = copy_rows(pop, row, p.pop0, (size_t)p.pitch * sizeof(float), row, (size_t)p.N, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && fit) e = cudaMemcpyAsync(fit, p.fit, fbytes, cudaMemcpyDeviceToHost, s);
+  if (e != cudaSuccess) cudaGetLastError();        // a refused copy is this call's error alone
   return e;
 }
 
@@ -232,6 +268,7 @@ cudaError_t rows_from_host(const GenParams& p, int parity, const float* pop, con
   if (e == cudaSuccess)
     e = copy_rows(p.pop0, (size_t)p.pitch * sizeof(float), pop, row, row, (size_t)p.N, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && fit) e = cudaMemcpyAsync(p.fit, fit, fbytes, cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) cudaGetLastError();
   return e;
 }
 

@@ -96,18 +96,9 @@ inline cudaError_t copy_rows(void* dst, size_t dpitch, const void* src, size_t s
   if (dpitch == width && spitch == width) return cudaMemcpyAsync(dst, src, width * rows, kind, s);
   return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, kind, s);
 }
-// Whether a kernel may address all of a host buffer: page-locked and mapped at
-// both ends, on a 16-byte boundary.
-inline bool mapped_host(const void* ptr, size_t bytes) {
-  if (!ptr || ((uintptr_t)ptr & 15u) != 0 || bytes == 0) return false;
-  cudaPointerAttributes a, b;
-  const void* end = static_cast<const char*>(ptr) + bytes - 1;
-  const bool ok = cudaPointerGetAttributes(&a, ptr) == cudaSuccess && a.type == cudaMemoryTypeHost &&
-                  a.devicePointer == ptr && cudaPointerGetAttributes(&b, end) == cudaSuccess &&
-                  b.type == cudaMemoryTypeHost && b.devicePointer == end;
-  cudaGetLastError();
-  return ok;
-}
+// Whether a kernel may address all of a host buffer: page-locked and mapped from
+// end to end, on a 16-byte boundary (api.cu).
+bool mapped_host(const void* ptr, size_t bytes);
 // The current rows and their fitness to host memory, and a population (with its
 // fitness, or without) from it into buffer 0, where every row of the generation
 // of this parity then lies.
