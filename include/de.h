@@ -185,8 +185,9 @@ int de_step(de_ctx *ctx);
  * (on the first run of that count, or by de_prepare_run) and replayed; a
  * setter that changes the launch (kernel, launch shape, pipeline, base rule,
  * wait limit) drops the cached graphs. Populations that the GPU's shared
- * memory holds advance many generations per launch, with the results of
- * de_step bit for bit; the first such run takes two more population buffers
+ * memory holds advance many generations per launch where the run is long enough
+ * to pay for it (from 2 to 8 generations on, by shape and crossover), with the
+ * results of de_step bit for bit; the first such run takes two more population buffers
  * from the allocator (without them, and on a capturing stream, every
  * generation is a launch). The waits between rows in that launch give up
  * after 1 s or the limit that de_set_wait_limit gives (DE_ETIMEOUT). */

@@ -470,20 +470,20 @@ int de_step(de_ctx* c) {
   return rc;
 }
 
-// Whether runs of this context go through the resident kernel: rows of the
-// row-per-CTA kernel chosen automatically, a base rule that needs nothing from
-// the previous generation's close, and a population that the chip holds. The
-// first such run takes the kernel's buffers; if that fails, runs launch each
-// generation.
-static bool resident_ready(de_ctx* c, ResidentShape* shape) {
+// Whether a run of this many generations goes through the resident kernel: rows of
+// the row-per-CTA kernel chosen automatically, a base rule that needs nothing from
+// the previous generation's close, a population that the chip holds and generations
+// enough to pay for the launch. The first such run takes the kernel's buffers; if
+// that fails, runs launch each generation.
+static bool resident_ready(de_ctx* c, int32_t generations, ResidentShape* shape) {
   if (c->batch || c->rotated || c->use_pipe || c->use_stream || c->kernel_req != 0) return false;
   if (c->p.base == kBaseBest) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-  shape->cluster = prepare_cluster(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR);
+  shape->cluster = prepare_cluster(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR, generations);
   const bool ok = shape->cluster ||
-                  prepare_resident(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR, c->sm_count,
-                                   c->smem_optin, shape);
+                  prepare_resident(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR, generations,
+                                   c->sm_count, c->smem_optin, shape);
   cudaGetLastError();
   if (!ok) return false;
   if (c->res_state) return true;
@@ -516,7 +516,7 @@ static cudaGraphExec_t run_graph(de_ctx* c, int32_t generations) {
   auto it = c->graphs.find(generations);
   if (it != c->graphs.end()) return it->second;
   ResidentShape shape;
-  const bool resident = resident_ready(c, &shape), segments = c->batch && batch_seg_ready(c, generations);
+  const bool resident = resident_ready(c, generations, &shape), segments = c->batch && batch_seg_ready(c, generations);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return nullptr;

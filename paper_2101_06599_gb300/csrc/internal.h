@@ -78,11 +78,11 @@ struct ResidentShape {
   size_t smem;
   bool cluster;                // gen_cluster.cu instead (the rest then says nothing)
 };
-// The launch shape for rows of block x kVecChoices[vidx] slots, and the
-// kernel's attributes set for it; false if the population does
-// not fit or a launch per generation is the faster.
-bool prepare_resident(int xo, int obj, int vidx, int block, int N, int D4, double CR, int sm_count, int smem_optin,
-                      ResidentShape* out);
+// The launch shape for a run of `gens` generations on rows of block x
+// kVecChoices[vidx] slots, and the kernel's attributes set for it; false if the
+// population does not fit or a launch per generation is the faster.
+bool prepare_resident(int xo, int obj, int vidx, int block, int N, int D4, double CR, int gens, int sm_count,
+                      int smem_optin, ResidentShape* out);
 cudaError_t launch_resident(int xo, int obj, int vidx, const ResidentShape& sh, ResidentParams rp, cudaStream_t s);
 // seg: the kernel that computes what a segment changed, else whole rows
 const void* resident_entry_sphere(bool seg, int vidx);
@@ -94,7 +94,7 @@ const void* resident_entry_elliptic(bool seg, int vidx);
 
 // The same for small populations, in one cluster (gen_cluster.cu). hist: the
 // ResState's, all ones between launches.
-bool prepare_cluster(int xo, int obj, int vidx, int block, int N, int D4, double CR);
+bool prepare_cluster(int xo, int obj, int vidx, int block, int N, int D4, double CR, int gens);
 cudaError_t launch_cluster(int xo, int obj, const GenParams& p, int gens, unsigned long long* hist, cudaStream_t s);
 
 // Batched instances (batch_kernel.cu): one descriptor per instance and a
