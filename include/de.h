@@ -186,7 +186,7 @@ int de_step(de_ctx *ctx);
  * setter that changes the launch (kernel, launch shape, pipeline, base rule,
  * wait limit) drops the cached graphs. Populations that the GPU's shared
  * memory holds advance many generations per launch where the run is long enough
- * to pay for it (from 2 to 8 generations on, by shape and crossover), with the
+ * to pay for it (from 2 to 5 generations on, by shape and crossover), with the
  * results of de_step bit for bit; the first such run takes two more population buffers
  * from the allocator (without them, and on a capturing stream, every
  * generation is a launch). The waits between rows in that launch give up

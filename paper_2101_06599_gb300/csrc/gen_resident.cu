@@ -34,21 +34,18 @@ static int sums_of(int obj) {
 // Populations that shared memory does not hold launch each generation.
 //
 // The fewest generations that pay for the launch, which loads the rows, forms every
-// sum and writes all back (us per run, Rastrigin, resident / a launch each):
-//  - segments: four (N = 250, D = 30, NEC at 3 and 4 generations 18.5 / 18.5, 20.6 /
-//    22.6; N = 1024, D = 1000 22.6 / 20.6, 25.2 / 26.8). Three with eight rows per CTA
-//    or more, where a launch costs more (N = 2000, D = 64 at 2 and 3: 16.5 / 16.5, 19.7 /
-//    22.7; N = 5000, D = 30 28.6 / 27.4, 35.0 / 38.9). Five with one row per CTA and
-//    more than 128 slots (N = 64, D = 1000 at 4 and 8: 22.7 / 20.6, 33.0 / 39.0), and
-//    where one warp walks for many rows (exponential, Cr = 0.9, N = 5000, D = 120 at
-//    3, 4 and 8: 46.8 / 40.5, 54.8 / 51.8, 85.2 / 98.2).
-//  - binomial rows of one warp: four up to 16 slots (N = 1000, D = 30 at 3 and 4: 18.5 /
-//    18.5, 20.9 / 22.7), else five (N = 2000, D = 128 at 4 and 8: 32.6 / 28.8, 42.4 / 53.4).
-//    Of several warps: eight (N = 300, D = 500 at 4, 8 and 16: 28.8 / 22.6, 40.4 / 40.8,
-//    58.4 / 76.3; N = 300, D = 1500 36.4 / 26.7, 49.2 / 48.7, 77.3 / 93.4).
-static int least_generations(int xo, int nw, int rpc, int D4, double CR) {
-  if (xo == kBin) return nw > 1 ? 8 : (D4 > 16 ? 5 : 4);
-  if ((rpc == 1 && D4 > 128) || (xo == kExp && CR > 0.5 && rpc > 16)) return 5;
+// sum and writes all back: four (us per run of 3, 4, 8 generations, Rastrigin, resident /
+// a launch each: N = 250, D = 30 NEC 18.5 / 18.5, 20.6 / 22.8, 29.1 / 43.1; N = 1024, D =
+// 1000 22.6 / 20.6, 26.2 / 26.7, 36.3 / 49.2; binomial N = 300, D = 500 18.1 / 16.5, 20.4 /
+// 21.7, 29.0 / 40.7; N = 300, D = 1500 20.5 / 20.6, 24.5 / 26.5, 36.6 / 49.1). Three with
+// eight rows per CTA or more, where a launch costs more (at 2 and 3: N = 2000, D = 64 NEC
+// 16.7 / 16.5, 20.4 / 22.6, D = 128 binomial 16.1 / 15.9, 18.5 / 21.9). Five for segments
+// with one row per CTA and more than 128 slots (N = 64, D = 1000 at 4 and 5: 23.3 / 22.5,
+// 26.4 / 26.7), and where one warp walks for many rows (exponential, Cr = 0.9, N = 5000, D
+// = 120 at 4, 5 and 8: 54.0 / 51.0, 62.0 / 62.1, 84.1 / 96.2).
+static int least_generations(int xo, int rpc, int D4, double CR) {
+  if (xo != kBin && rpc == 1 && D4 > 128) return 5;
+  if (xo == kExp && CR > 0.5 && rpc > 16) return 5;
   return rpc >= 8 ? 3 : 4;
 }
 
@@ -62,7 +59,7 @@ bool prepare_resident(int xo, int obj, int vidx, int block, int N, int D4, doubl
   s.seg = xo != kBin;
   if (s.seg && (vidx != 0 || (D4 > 32 && (1.0 - CR) * 40.0 < 1.0))) return false;
   if (!s.seg && nw > 1 && s.rpc * nw > kResWarps) return false;
-  if (gens < least_generations(xo, nw, s.rpc, D4, CR)) return false;
+  if (gens < least_generations(xo, s.rpc, D4, CR)) return false;
   const int W = s.seg ? 1 : nw;
   // 15 named barriers, one per group of more than a warp
   s.groups = std::min(s.rpc, W > 1 ? std::min(kResWarps / W, 15) : kResWarps);

@@ -689,7 +689,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
   // the run's state: rows to buffer 0, fitness, slot bytes, counters; the last
   // CTA closes. Unless this CTA gave up, its second helper has seen every CTA
   // finish every generation, and nobody reads the buffers any more
-  if (masked) atomicAdd(&s_masked, masked);
+  masked = warp_sum_u64(masked);
+  if (masked && lane == 0) atomicAdd(&s_masked, masked);
   if (wins) atomicAdd(&s_wins, wins);
   if (key != ~0ULL) {
     atomicMin(&s_key, key);

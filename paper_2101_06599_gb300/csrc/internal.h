@@ -94,7 +94,7 @@ const void* resident_entry_elliptic(bool seg, int vidx);
 
 // The same for small populations, in one cluster (gen_cluster.cu). hist: the
 // ResState's, all ones between launches.
-bool prepare_cluster(int xo, int obj, int vidx, int block, int N, int D4, double CR, int gens);
+bool prepare_cluster(int xo, int obj, int vidx, int block, int N, int D4, double CR);
 cudaError_t launch_cluster(int xo, int obj, const GenParams& p, int gens, unsigned long long* hist, cudaStream_t s);
 
 // Batched instances (batch_kernel.cu): one descriptor per instance and a

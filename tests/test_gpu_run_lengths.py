@@ -9,10 +9,10 @@ from paper_2101_06599_gb300 import de as DE
 from paper_2101_06599_gb300 import workloads as W
 
 # the fewest generations on the chip: one cluster, rows of one warp and of several, one row per CTA, many
-LEAST = [(100, 30, "nec", 0.9, 2), (100, 30, "exp", 0.5, 3), (100, 30, "bin", 0.5, 3), (100, 100, "bin", 0.5, 5),
+LEAST = [(100, 30, "nec", 0.9, 2), (100, 30, "exp", 0.5, 2), (100, 30, "bin", 0.5, 2), (150, 128, "bin", 0.5, 2),
          (300, 500, "nec", 0.9, 4), (100, 30, "exp", 0.9, 4), (64, 1000, "nec", 0.9, 5), (2000, 64, "nec", 0.1, 3),
-         (5000, 30, "exp", 0.9, 5), (5000, 30, "exp", 0.5, 3), (1000, 30, "bin", 0.5, 4), (2000, 128, "bin", 0.5, 5),
-         (300, 500, "bin", 0.5, 8), (150, 2000, "bin", 0.5, 8)]
+         (5000, 30, "exp", 0.9, 5), (5000, 30, "exp", 0.5, 3), (1000, 30, "bin", 0.5, 4), (2000, 128, "bin", 0.5, 3),
+         (300, 500, "bin", 0.5, 4), (150, 2000, "bin", 0.5, 4)]
 
 
 @pytest.mark.parametrize("N,D,xo,cr,least", LEAST)
