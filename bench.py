@@ -190,14 +190,14 @@ def time_variant(DE, torch, N, D, xo, obj, steps, warmup, seed, ramp_s=0.0, samp
         raise
 
 
-def time_batched(DE, torch, steps, warmup, seed, peak, n_inst=None, kernels="tuned"):
+def time_batched(DE, torch, steps, warmup, seed, peak, n_inst=None, kernels="auto"):
     """The 512-instance workload (D log-uniform in [10, 2000], N = min(10 D,
     4096), sphere/Rastrigin/Ackley/Rosenbrock round-robin, NEC, F = 0.5,
     Cr = 0.9), one generation of every instance per step. n_inst keeps the
     first n_inst instances (a smaller case of the same mix, for profiling).
-    kernels: "tuned" (de_batch_autotune picks the row kernel per class of
-    instances), or every instance on the streaming ("flow") or the staged
-    ("staged") kernel."""
+    kernels: "auto" (what a run picks by itself), "tuned" (the row kernels that
+    de_batch_autotune picks per class of instances), or every instance on the
+    streaming ("flow") or the staged ("staged") kernel."""
     from paper_2101_06599_gb300 import workloads as Wk
     specs = [dict(N=s.N, D=s.D, obj=s.objective, bounds=Wk.BOXES[s.objective], xo="nec", CR=CR_DEF, F=F_DEF)
              for s in Wk.batched_specs()]
@@ -209,15 +209,18 @@ def time_batched(DE, torch, steps, warmup, seed, peak, n_inst=None, kernels="tun
     try:
         t_tune = time.time()
         if kernels == "tuned":
-            groups = b.autotune(reps=3)
-        else:
+            b.set_groups(b.autotune(reps=3))     # named, so that runs use them
+        elif kernels != "auto":
             b.set_groups([2 if kernels == "flow" else 1] * len(specs))
-            groups = b.groups()
+        groups = b.groups()
         t_tune = time.time() - t_tune
         def kind(g):
             return "staged" if g < 0 else ("streaming" if g == 2 else ("register" if g <= 32 else "cta"))
-        kinds = sorted({kind(g) for g in groups})
-        b.run(warmup)
+        kinds = [kind(g) for g in groups]
+        held = len(DE._live_blocks)
+        b.run(max(2, warmup))
+        if len(DE._live_blocks) > held:          # the first segment run takes its buffers
+            kinds = ["segments"] * len(specs)
         b.prepare_run(steps)
         b.synchronize()
         st0 = b.stats()
@@ -244,12 +247,14 @@ def time_batched(DE, torch, steps, warmup, seed, peak, n_inst=None, kernels="tun
     return {"workload": "batched_512_instances" if len(specs) == 512 else "batched_first_%d_instances" % len(specs),
             "instances": len(specs), "ind_dims_per_step": units,
             "value": units * steps / (ms / 1e3), "unit": UNIT, "ms_per_gen": ms / steps,
-            # a run keeps the rows' partial sums and touches only what the segments change, one
-            # launch per generation: the share that reading every row once would need
-            # at the copy rate, over 1 when a generation is faster than that
+            # segment runs keep the rows' partial sums and touch only what the segments change: the
+            # share of the copy rate that reading every row once would need, over 1 when a
+            # generation is faster than that
             "full_rows_share": gbs / peak,
-            "launches_per_step": 1,
-            "row_kernels": {kd: sum(1 for g in groups if kind(g) == kd) for kd in kinds},
+            # segments, or every instance staged or streaming: one launch per generation
+            "launches_per_step": 1 if len(set(kinds)) == 1 and kinds[0] in ("segments", "staged", "streaming")
+            else 2 + len(set(kinds)),
+            "row_kernels": {kd: kinds.count(kd) for kd in sorted(set(kinds))},
             "autotune_s": round(t_tune, 3),
             "a_acceptance": d_acc / (rows * steps), "m_masked_fraction": d_msk / (units * steps)}
 
@@ -655,8 +660,8 @@ def main():
     ap.add_argument("--no-small", action="store_true")
     ap.add_argument("--batch-instances", type=int, default=0,
                     help="batched leg: keep the first K of the 512 instances (profiling)")
-    ap.add_argument("--batch-kernels", default="tuned", choices=["tuned", "flow", "staged"],
-                    help="batched leg: row kernels picked by the autotuner, or one kernel for every instance")
+    ap.add_argument("--batch-kernels", default="auto", choices=["auto", "tuned", "flow", "staged"],
+                    help="batched leg: what a run picks, the autotuner's row kernels, or one kernel for every instance")
     ap.add_argument("--no-crossover", action="store_true")
     ap.add_argument("--no-table2", action="store_true")
     ap.add_argument("--only", choices=["rotated", "small", "batched", "crossover", "table2"],

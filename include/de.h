@@ -327,8 +327,8 @@ typedef struct {
  * cooperative kernel launch (draws, rows, close) when every instance is on
  * the staged kernel (the default for exp / NEC rows of D <= 2048), else a
  * few launches over all instances (draws, row kernels, close). A de_run of
- * two or more generations on exp / NEC rows of D <= 2048 (1 / (1 - Cr) <= 60,
- * no wait limit set) keeps the rows' partial sums for the run and touches only
+ * two or more generations on exp / NEC rows of D <= 2048 (1 / (1 - Cr) <= 60 or
+ * D <= 32, no wait limit set, no kernels named by de_batch_set_groups) keeps the rows' partial sums for the run and touches only
  * what the segments change, with the same results bit for bit; the first such
  * run takes 128 to 384 bytes per row from the allocator (without them the run
  * reads every row). The rows of
@@ -384,12 +384,17 @@ int de_batch_debug_step(de_ctx *ctx, int32_t inst, float *trial_out, float *ftri
  * the choice, and so are fitness values, selections and trajectories for
  * every choice with at most 32 threads per row (staged, streaming, and
  * G = 4..32): those kernels sum the FP32 fitness in one fixed order. G > 32 (needed only
- * for D > 2048) sums in another order. Returns DE_EINVAL for an invalid
+ * for D > 2048) sums in another order. A value other than 0 for any instance
+ * holds for the batch's runs too: they launch these kernels each generation and
+ * do not keep partial sums (de_batch_create); all zeros, or de_batch_autotune,
+ * leave runs to the library again. Returns DE_EINVAL for an invalid
  * value; the context is unchanged then. */
 int de_batch_set_groups(de_ctx *ctx, const int32_t *groups);
 int de_batch_get_groups(de_ctx *ctx, int32_t *groups);
 
-/* Autotuner: pick each instance's row kernel (the values above) by timing.
+/* Autotuner: pick each instance's row kernel (the values above) by timing, for
+ * single generations and the runs that do not keep partial sums (pass the choice
+ * to de_batch_set_groups for all runs to use it).
  * Instances are grouped by crossover and the octave of ceil(D/4) (rows of
  * D <= 2048; wider rows keep their tiles). For each group in turn, every
  * candidate (register tiles of 4..32 lanes per row; for exp and NEC the

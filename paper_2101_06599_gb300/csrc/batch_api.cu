@@ -196,9 +196,10 @@ cudaError_t batch_launch_generation(de_ctx* c, bool, int) {
 // generation in runs of 2, 4, 100: 314, 236, 164 against 568, 554, 559) and while
 // 1 / (1 - Cr) <= 60 genes (Cr = 0.95 252 / 572, 0.97 362 / 589, 0.98 462 / 627;
 // longer segments come near to every slot) or rows have at most 8 slots. A batch
-// whose wait limit was set keeps the kernel with the wait.
+// whose wait limit was set keeps the kernel with the wait, one whose row kernels
+// were named by de_batch_set_groups keeps to those.
 bool batch_seg_ready(de_ctx* c, int generations) {
-  if (generations < 2 || c->wait_ns != 0ull) return false;
+  if (generations < 2 || c->wait_ns != 0ull || c->bchosen) return false;
   int ns = 1;
   for (int k = 0; k < c->n_inst; ++k) {
     const int D4 = c->bp[k].D4;
@@ -597,6 +598,7 @@ int de_batch_set_groups(de_ctx* c, const int32_t* groups) {
   if (sync_stream(c) != DE_OK) return DE_ECUDA;
   c->bgroup = g;
   c->blanes = l;
+  c->bchosen = std::any_of(groups, groups + c->n_inst, [](int32_t v) { return v != 0; });
   return build_tiles(c);
 }
 
@@ -752,6 +754,7 @@ int de_batch_autotune(de_ctx* c, int32_t reps, int32_t* groups_out) {
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   ctx_free(c, snap);
+  c->bchosen = false;
   const int rb = build_tiles(c);
   if (rc == DE_OK) rc = rb;
   if (rc == DE_OK && groups_out) rc = de_batch_get_groups(c, groups_out);

@@ -78,6 +78,7 @@ struct de_ctx {
   de::DevState* d_states = nullptr;
   int nctiles = 0, batch_grid = 0, max_pitch = 0;
   de::BatchSeg bseg{};                   // segment runs (made by the first one)
+  bool bchosen = false;                  // de_batch_set_groups named a kernel, which runs keep to
   // shifted-rotated objectives (sr_api.cu)
   bool rotated = false;
   de::SrParams sp{};
