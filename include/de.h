@@ -188,7 +188,8 @@ int de_step(de_ctx *ctx);
  * memory holds advance many generations per launch where the run is long enough
  * to pay for it (from 2 to 5 generations on, by shape and crossover), with the
  * results of de_step bit for bit; the first such run takes two more population buffers
- * from the allocator (without them, and on a capturing stream, every
+ * and 128 bytes a row from the allocator, 256 bytes in all where one cluster of
+ * SMs holds the rows (without them, and on a capturing stream, every
  * generation is a launch). The waits between rows in that launch give up
  * after 1 s or the limit that de_set_wait_limit gives (DE_ETIMEOUT). */
 int de_run(de_ctx *ctx, int32_t generations);

@@ -486,25 +486,32 @@ static bool resident_ready(de_ctx* c, int32_t generations, ResidentShape* shape)
                                    c->sm_count, c->smem_optin, shape);
   cudaGetLastError();
   if (!ok) return false;
-  if (c->res_state) return true;
-  ResState* rs = (ResState*)ctx_alloc(c, sizeof(ResState));
+  if (!c->res_state) {
+    ResState* rs = (ResState*)ctx_alloc(c, sizeof(ResState));
+    // row words and counters start at tag 0, the first launch at tag 8: no word
+    // is taken for one of its generations before its owner has written it
+    ResState s0;
+    std::memset(&s0, 0, sizeof(s0));
+    s0.epoch = 8u;
+    s0.hist = ~0ULL;
+    if (!rs || cudaMemcpyAsync(rs, &s0, sizeof(s0), cudaMemcpyHostToDevice, c->stream) != cudaSuccess) {
+      cudaGetLastError();
+      if (rs) ctx_free(c, rs);
+      return false;
+    }
+    c->res_state = rs;
+  }
+  if (shape->cluster || c->res_words) return true;   // one cluster keeps its rows on the chip
   uint32_t* words = (uint32_t*)ctx_alloc(c, (size_t)c->N * kResWordStride * sizeof(uint32_t));
   float* pop2 = (float*)ctx_alloc(c, 2 * (size_t)c->N * (size_t)c->pitch * sizeof(float));
-  // row words and counters start at tag 0, the first launch at tag 8: no word
-  // is taken for one of its generations before its owner has written it
-  ResState s0;
-  std::memset(&s0, 0, sizeof(s0));
-  s0.epoch = 8u;
-  s0.hist = ~0ULL;
-  if (rs && words && pop2 && cudaMemcpyAsync(rs, &s0, sizeof(s0), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
+  if (words && pop2 &&
       cudaMemsetAsync(words, 0, (size_t)c->N * kResWordStride * sizeof(uint32_t), c->stream) == cudaSuccess) {
-    c->res_state = rs;
     c->res_words = words;
     c->res_pop2 = pop2;
     return true;
   }
   cudaGetLastError();
-  for (void* q : {(void*)rs, (void*)words, (void*)pop2})
+  for (void* q : {(void*)words, (void*)pop2})
     if (q) ctx_free(c, q);
   return false;
 }

@@ -44,7 +44,8 @@ struct de_ctx {
   size_t pipe_smem = 0;
   int sm_count = 0, smem_optin = 0;
   GenParams p{};
-  ResState* res_state = nullptr;   // resident runs: state, row words, two more row buffers (made by the first run)
+  ResState* res_state = nullptr;   // resident runs: state and, but for one cluster, row words and two more row
+                                   // buffers (made by the first run)
   uint32_t* res_words = nullptr;
   float* res_pop2 = nullptr;
   std::vector<de_host::Block> blocks;

@@ -126,7 +126,8 @@ int sr_setup(de_ctx* c, const de_objparams* prm) {
   float* shift = (float*)ctx_alloc(c, (size_t)D * sizeof(float));
   float* rot = (float*)ctx_alloc(c, (size_t)D * D * sizeof(float));
   sp.part_g = (float*)ctx_alloc(c, (size_t)N * sp.nct * sizeof(float));
-  sp.part_w = (float*)ctx_alloc(c, (size_t)N * sp.nct * sizeof(float));
+  const bool want_w = sp.prec != 0 && prm->bound == DE_BOUND_WORST_CASE;   // who reads the sums of w |z|
+  if (want_w) sp.part_w = (float*)ctx_alloc(c, (size_t)N * sp.nct * sizeof(float));
   sp.norm2 = (float*)ctx_alloc(c, (size_t)N * sizeof(float));
   sp.amax = (float*)ctx_alloc(c, (size_t)N * sizeof(float));
   sp.fit_err = (float*)ctx_alloc(c, (size_t)N * sizeof(float));
@@ -137,7 +138,7 @@ int sr_setup(de_ctx* c, const de_objparams* prm) {
   sp.inc_count = (unsigned*)ctx_alloc(c, sizeof(unsigned));
   sp.finish_due = (int*)ctx_alloc(c, sizeof(int));
   sp.inc_every = c->incumbent_every;
-  if (!shift || !rot || !sp.part_g || !sp.part_w || !sp.norm2 || !sp.amax || !sp.fit_err || !sp.amb || !sp.amb_count ||
+  if (!shift || !rot || !sp.part_g || (want_w && !sp.part_w) || !sp.norm2 || !sp.amax || !sp.fit_err || !sp.amb || !sp.amb_count ||
       !sp.part2_g || !sp.inc_part || !sp.inc_count || !sp.finish_due)
     return DE_ENOMEM;
   sp.shift = shift;

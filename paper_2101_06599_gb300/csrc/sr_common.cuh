@@ -30,7 +30,7 @@ struct SrParams {
   uint16_t* a_lo;          // lo(u - o): the rounded remainder, N x D
   float* part_g;           // N x nct: sum of g(z) over the column tile
   float* part_w;           // N x nct: sum of w_k |z_k| (w = 1 Rastrigin, c_k elliptic), split products
-                           // with the worst-case bound
+                           // with the worst-case bound alone (else null)
   float* norm2;            // N: |u - o|^2 of the trial (FP32)
   float* amax;             // N: max_j |u_j - o_j| of the trial
   float* fit_err;          // N: bound on |fit - FP32-path value| of the stored parent
