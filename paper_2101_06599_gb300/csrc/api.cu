@@ -243,8 +243,12 @@ bool mapped_host(const void* ptr, size_t bytes) {
 // 3409, 128 instances (760 MB) 7.15 -> 5.78 ms.
 // Anything else goes through the copy engine.
 // Populations from the host of more than this go by one linear copy where their
-// rows allow it: the kernel's first reads of that much host memory are slower (655
-// MB and 20 generations 6.28 ms with it, 6.23 with the copy).
+// rows allow it. us, copy / kernel, for a buffer's first use and repeated: 4 MB 69 / 63,
+// 44 / 42; 17 MB 137 / 137, 106 / 103; 34 MB 240 / 236, 188 / 186; 67 MB 427 / 432, 354 /
+// 349; 101 MB 585 / 609, 518 / 514; 134 MB 772 / 812, 681 / 680; 268 MB 1430 / 1410, 1340 /
+// 1336. Jobs with 20 generations, repeated: 34 MB 832 / 824, 134 MB 2228 / 2226, 268 MB
+// 3153 / 3157, 655 MB 5997 / 6000, and with new buffers (bench.py) 6240 / 6300. So the
+// kernel's first reads cost more from about 64 MB on, and above 200 MB it gains nothing.
 constexpr size_t kCopyInBytes = 64u << 20;
 
 cudaError_t rows_to_host(const GenParams& p, float* pop, float* fit, cudaStream_t s) {
