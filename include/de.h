@@ -189,8 +189,9 @@ int de_step(de_ctx *ctx);
  * to pay for it (from 2 to 5 generations on, by shape and crossover), with the
  * results of de_step bit for bit; the first such run takes two more population buffers
  * and 128 bytes a row from the allocator, 256 bytes in all where one cluster of
- * SMs holds the rows (without them, and on a capturing stream, every
- * generation is a launch). The waits between rows in that launch give up
+ * SMs holds the rows (without them every generation is a launch). While the
+ * stream is being captured, a count that has no graph yet is refused (DE_ECUDA,
+ * as by de_prepare_run; the capture and the context go on). The waits between rows in that launch give up
  * after 1 s or the limit that de_set_wait_limit gives (DE_ETIMEOUT). */
 int de_run(de_ctx *ctx, int32_t generations);
 

@@ -530,7 +530,10 @@ static cudaGraphExec_t run_graph(de_ctx* c, int32_t generations) {
   const bool resident = resident_ready(c, generations, &shape), segments = c->batch && batch_seg_ready(c, generations);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) return nullptr;
+  if (e != cudaSuccess) {                          // the stream is being captured: an error of this call alone
+    cudaGetLastError();
+    return nullptr;
+  }
   cudaError_t le = cudaSuccess;
   if (resident) {
     ResidentParams rp{};

@@ -2,7 +2,8 @@
 thread 1 to 16, one warp to 16, more rows than the GPU holds CTAs, alone, in chains
 and replayed from a captured graph. It sums as the row-per-CTA kernel of a context
 does, so rows and values are that kernel's bit for bit (tolerance zero)."""
-import numpy as np
+import gc
+
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -64,6 +65,7 @@ def test_captured_chain(N, D):
     _call(x, f, N, D, pitch, 0.8, obj, box, 7, 0, torch.cuda.current_stream().cuda_stream)   # the thresholds
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph()
+    gc.collect()                                 # a graph of an earlier test may not end while this one is captured
     with torch.cuda.graph(graph):
         for g in range(4):
             _call(x, f, N, D, pitch, 0.8, obj, box, 7, g, torch.cuda.current_stream().cuda_stream)

@@ -1,6 +1,8 @@
 """Short runs: below the generations that pay for an on-chip launch a run launches
 each generation and takes no buffers; whatever the count, the results are those of
 single generations, bit for bit (tolerance zero)."""
+import gc
+
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -31,3 +33,32 @@ def test_fewest_generations_on_the_chip(N, D, xo, cr, least):
         assert a.stats() == c.stats()
         a.close()
         c.close()
+
+
+@pytest.mark.parametrize("N,D", [(100, 30), (300, 500), (64, 3000)])
+def test_a_run_without_a_graph_is_refused_under_capture(N, D):
+    import torch
+    kw = dict(obj="sphere", bounds=(-5.0, 5.0), seed=1)
+    o, ref = DE.Optimizer(N, D, **kw), DE.Optimizer(N, D, **kw)
+    o.run(3)
+    o.synchronize()
+    y = torch.zeros(4, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    gc.collect()                                 # a graph of an earlier test may not end while this one is captured
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=o.stream):
+        y.add_(1)
+        for call in (o.run, o.prepare_run):
+            with pytest.raises(DE.DEError) as e:
+                call(7)
+            assert e.value.code == DE.DE_ECUDA
+        y.add_(1)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert y.tolist() == [2.0] * 4
+    o.run(7)                                     # the context goes on
+    ref.run(10)
+    for u, v in zip(o.population(), ref.population()):
+        assert u.tobytes() == v.tobytes()
+    o.close()
+    ref.close()
