@@ -12,8 +12,8 @@
 //
 // Nothing goes through L2 between the first and the last generation, where the
 // resident kernel (gen_resident.cuh) pays three round trips and a fence each:
-// NEC sphere N = 100, D = 30 2.3 us per generation there (4.8 us with a launch each),
-// 1.1 us here, of which a cluster barrier is 0.28 us. What is left is the chain of
+// NEC sphere N = 100, D = 30 2.0 us per generation there (4.5 us with a launch each),
+// 1.0 us here, of which a cluster barrier is 0.28 us. What is left is the chain of
 // about 200 dependent instructions.
 // Sums run in gen_kernel's order, so results are de_step's bit for bit.
 #include <algorithm>
@@ -268,12 +268,13 @@ cudaLaunchConfig_t config(int N, cudaLaunchAttribute* attr, cudaStream_t s) {
 }  // namespace
 
 // Where the cluster is the faster (us per generation, cluster against resident):
-// NEC up to its 248 rows (N = 100, D = 30 1.1 / 2.3, N = 248, D = 128, Ackley 2.1 /
-// 2.7). Binomial up to 160 rows, or shorter ones (Ackley, D = 128: N = 60 1.6 /
-// 2.4, N = 150 2.4 / 2.5, N = 248 3.3 / 3.1; N = 248, D = 60 2.2 / 3.2): beyond, 8
-// SMs have too many genes to draw and sum. Exponential while its walk is short: one
-// warp walks for all rows of a CTA (D = 128, N = 248: Cr = 0.3 2.2 / 2.4, 0.9 6.6 /
-// 2.5).
+// NEC up to its 248 rows (N = 100, D = 30 1.0 / 2.0, N = 248, D = 128, Ackley 2.1 /
+// 2.6). Binomial up to 160 rows, or shorter ones (Ackley, D = 128: N = 60 1.5 /
+// 2.3, N = 130 2.1 / 2.3, N = 160 2.3 / 2.3, N = 200 2.8 / 2.3; D = 60: N = 200 2.3 / 2.4,
+// N = 248 2.5 / 2.4; D = 30: N = 248 2.3 / 2.4): beyond, 8 SMs have too many genes to
+// draw and sum. Exponential while its walk is short: one warp walks for all rows of a
+// CTA (D = 128, N = 248: Cr = 0.3 2.4 / 2.5, 0.5 2.3 / 2.2, 0.9 6.5 / 2.2; N = 130, D = 60,
+// Cr = 0.5 1.8 / 2.1).
 // From two generations on it is not the slower (us per run of 2, 3, 4 generations,
 // Rastrigin, cluster / a launch each: N = 100, D = 30 NEC 8.5 / 12.3, 10.3 / 18.5, 12.3 /
 // 22.6; N = 248, D = 128, exponential, Cr = 0.5 12.6 / 12.6, 16.4 / 18.5, 17.9 / 22.6; N =

@@ -25,12 +25,13 @@ static int sums_of(int obj) {
 // the sizes named, us per generation, resident against a launch each):
 //  - exp and NEC: one slot per thread (D <= 1024) and segments that mostly fit
 //    a slot per lane, 1 / (1 - Cr) <= 40 genes or rows of at most 32 slots.
-//    N = 1024, D = 1000: Cr = 0.9 3.0 / 5.9, Cr = 0.95 (exp) 3.4 / 12.9, Cr =
-//    0.99 5.4 / 5.8, Cr = 0.999 9.5 / 6.0; two slots per thread, N = 300, D =
-//    1100: 6.9 / 5.3.
-//  - binomial: rows of one warp (N = 5000, D = 128 7.7 / 11.5), or all rows of
-//    a CTA at once: N = 600, D = 500 (16 warps) 4.7 / 6.2, N = 800 (24 warps)
-//    6.2 / 5.0.
+//    N = 1024, D = 1000: Cr = 0.9 2.5 / 5.7, Cr = 0.95 (exp) 2.6 / 12.8, Cr =
+//    0.975 2.8 / 5.7, 0.99 3.8 / 5.7, 0.999 7.0 / 6.0 (the line is on the safe side); two
+//    slots per thread lose (N = 300, D = 1100 6.9 / 5.3).
+//  - binomial: rows of one warp (N = 5000, D = 128 7.0 / 11.5), or all rows of
+//    a CTA at once: N = 600, D = 500 (16 warps) 2.6 / 5.0. Beyond, a CTA's rows take
+//    turns: N = 700 (20 warps) 4.6 / 4.9, N = 500, D = 1000, Ackley (32) 5.2 / 5.4, N =
+//    1024, D = 1000 (56) 9.0 / 7.4.
 // Populations that shared memory does not hold launch each generation.
 //
 // The fewest generations that pay for the launch, which loads the rows, forms every

@@ -48,10 +48,12 @@
 // What bounds it: latency. A generation is the chain poll a word (L2, 0.5 us on
 // a line that another SM has just written), load the genes (0.5 us), some 300
 // dependent instructions, fence and publish (0.5 us). Per generation, against
-// a launch each: NEC sphere N = 100, D = 30 4.8 -> 2.3 us, Rastrigin N = 1024,
-// D = 1000 5.9 -> 3.0 us (exponential at Cr = 0.5 7.1 -> 2.8 us), binomial
-// Griewank N = 300, D = 500 5.5 -> 3.4 us. Words that share a line cost twice
-// that (5 us at N = 300, D = 500): each has a line of its own.
+// a launch each: NEC sphere N = 100, D = 30 4.5 -> 2.0 us, Rastrigin N = 1024,
+// D = 1000 5.7 -> 2.5 us (exponential at Cr = 0.5 6.6 -> 2.5 us), binomial
+// Griewank N = 300, D = 500 5.5 -> 2.9 us. Words that share a line cost twice
+// that (5 us at N = 300, D = 500): each has a line of its own. Waits that let the
+// lanes of a warp leave one by one cost up to twice as well, for as long as the lanes
+// stayed apart: the same binomial run took 3.05 or 6.04 us from one launch to the next.
 #pragma once
 #include "draws.cuh"
 #include "internal.h"
@@ -133,7 +135,7 @@ __host__ __device__ inline ResLayout res_layout(bool seg, int rpc, int D4, int g
 }
 
 // One slot q of a row (genes 4q ..) added to a thread's sums; nb is gene 4q + 4.
-template <bool kSeg, int OBJ>
+template <int OBJ>
 __device__ __forceinline__ void res_slot(Acc& a, const float4& x, float nb, int q, const GenParams& p) {
   const int j0 = 4 * q;
   if constexpr (OBJ == kRosenbrock) {
@@ -141,7 +143,7 @@ __device__ __forceinline__ void res_slot(Acc& a, const float4& x, float nb, int 
     if (j0 + 2 < p.D) accum_pair(a, x.y, x.z);
     if (j0 + 3 < p.D) accum_pair(a, x.z, x.w);
     if (j0 + 4 < p.D) accum_pair(a, x.w, nb);
-  } else if constexpr (kSeg && OBJ == kGriewank) {
+  } else if constexpr (OBJ == kGriewank) {
     griewank_slot(a, x, j0, p);
   } else {
     accum_gene<OBJ>(a, x.x, j0, p);
@@ -391,7 +393,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         if constexpr (OBJ == kRosenbrock) {
           if (q + 1 < p.D4) nb = ((q + 1 >= a0 && q + 1 <= b0) || q + 1 <= b1) ? tr[q + 1].x : x[q + 1].x;
         }
-        res_slot<kSeg, OBJ>(s, xv, nb, q, p);
+        res_slot<OBJ>(s, xv, nb, q, p);
       }
       to[32 * w + lane] = s.a;
       if (NS > 1) to[T + 32 * w + lane] = s.b;
@@ -470,13 +472,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
             if (lane == n0 - 1 || lane >= n - 1) nx = qe + 1 < p.D4 ? x[qe + 1].x : 0.0f;
             if (lane == n - 1 && qe + 1 == a0) nx = tx0;   // the slots after the wrap end where the first one begins
           }
-          // all lanes compute on. The shuffle is a meeting point that the compiler
-          // keeps here: without it (Rosenbrock has its own) the lanes outside the
-          // segment run the rest of the row's code apart, 3.9 us per generation
-          // against 2.4 at N = 50, D = 10, and a __syncwarp alone does not help
-          if constexpr (OBJ != kRosenbrock) (void)__shfl_down_sync(0xFFFFFFFFu, te.x, 1);
-          __syncwarp();
-          res_slot<kSeg, OBJ>(es, te, nx, qe, p);
+          __syncwarp();                            // all lanes compute on
+          res_slot<OBJ>(es, te, nx, qe, p);
           __syncwarp();
 #pragma unroll 1
           for (uint32_t todo = pl.again; todo; todo &= todo - 1u) {
@@ -637,7 +634,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
             if (lane == 31) nb = (pw + 1 < nw) ? first[v * 8 + pw + 1] : (v + 1 < V ? first[(v + 1) * 8] : 0.0f);
           }
           const int q = pw * 32 + lane + v * T;
-          if (q < p.D4) res_slot<kSeg, OBJ>(s, x[v], nb, q, p);
+          if (q < p.D4) res_slot<OBJ>(s, x[v], nb, q, p);
         }
         res_butterfly<NS, 16>(s);
         if (W > 1) {

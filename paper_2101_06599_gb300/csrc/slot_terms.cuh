@@ -8,12 +8,10 @@ namespace de {
 // Griewank: accum_gene of the genes j0 .. j0 + 3, each term by the same operations
 // and added in the same order, but the four terms side by side and both logarithms
 // in place of a branch per gene: one latency of sine and logarithm instead of four.
-// us per generation, branches -> this: segment rows NEC N = 300, D = 500 3.37 -> 2.89,
-// N = 1000, D = 1000 4.17 -> 3.70; one cluster N = 50, D = 30 NEC 1.98 -> 1.55, N = 100,
-// D = 50 binomial 2.50 -> 2.18, N = 200, D = 30 exponential (bound by the walk) 3.16 -> 3.18.
-// Where all lanes of many warps sum every slot, the operations count instead
-// (binomial N = 300, D = 500 3.33 -> 3.62 us per generation), so binomial rows keep
-// the branches.
+// us per generation, branches -> this: segment rows NEC N = 300, D = 500 3.17 -> 2.75,
+// N = 1000, D = 1000 3.57 -> 3.05; binomial rows N = 300, D = 500 3.23 -> 2.88, N = 600, D
+// = 100 2.89 -> 2.70; one cluster N = 50, D = 30 NEC 1.70 -> 1.46, N = 100, D = 50 binomial
+// 2.18 -> 2.13, N = 200, D = 30 exponential (bound by the walk) 2.96 -> 3.19.
 __device__ __forceinline__ void griewank_slot(Acc& a, const float4& x, int j0, const GenParams& p) {
   const float v[4] = {x.x, x.y, x.z, x.w};
   float t[4], n[4];
