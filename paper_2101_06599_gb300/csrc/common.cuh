@@ -85,8 +85,9 @@ struct GenParams {
 // every CTA of that kernel has called griddep_launch_dependents or exited):
 // its launch overlaps the previous kernel's tail instead of following it.
 // griddep_wait blocks until the previous kernel has completed and its memory
-// is visible; every kernel launched this way calls it before it reads or
-// writes anything. Both are no-ops for a kernel launched without it.
+// is visible; every kernel launched this way calls it before it reads what an
+// earlier kernel wrote or writes to global memory (barriers, tensor memory, draws and
+// what else needs neither may come first). Both are no-ops for a kernel launched without it.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

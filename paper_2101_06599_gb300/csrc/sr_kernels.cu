@@ -503,7 +503,7 @@ __device__ __forceinline__ void ls_items(const SrParams& sp, float* ls_smem, con
       cp_async_commit();
       const int st = step % kLsStages;
 #pragma unroll
-      for (int kk = lane; kk < kLsK; kk += 32) {   // a = fl(x - o): k = kk, the warp's 4 entries
+      for (int kk = lane; kk < kLsK; kk += 32) {   // a = fl(x - o): k = kk, the warp's WE entries
         const float* xs = Xs + (st * kLsE + ebase) * kLsLdX + kk;
         const float o = Os[st * kLsK + kk];
 #pragma unroll
